@@ -636,23 +636,6 @@ __global__ void hrt_gather_kernel(int nx, int ny, long long nfaces, const double
   y[t] = z[e1 * NL4 + f1 * NL + tt] + z[e2 * NL4 + f2 * NL + tt];
 }
 
-// row (f NL + tt) of H_e applied to the element's multipliers (boundary faces carry none)
-template <int P>
-__device__ __forceinline__ double he_row(int nx, int ny, const double* __restrict__ He,
-                                         const double* __restrict__ x, long long e, int f, int tt) {
-  constexpr int NL = P + 1, NL4 = 4 * NL;
-  const double* row = He + (size_t)e * NL4 * NL4 + (size_t)(f * NL + tt) * NL4;
-  double s = 0.0;
-#pragma unroll
-  for (int g = 0; g < 4; ++g) {
-    const long long fi = face_index(nx, ny, (int)e, g);
-    if (fi < 0) continue;
-#pragma unroll
-    for (int u = 0; u < NL; ++u) s = fma(row[g * NL + u], x[fi * NL + u], s);
-  }
-  return s;
-}
-
 // Element-patch additive Schwarz preconditioner: for each element the restriction of H to
 // the multipliers of its interior faces, H_e plus, on each such face, the neighbour's
 // diagonal block of that face (its only contribution there), inverted; the preconditioner
@@ -785,28 +768,36 @@ __global__ void hrt_recover_kernel(long long E, int nx, int ny, const double* __
 }
 
 // ---- the multiplier system's Krylov solve: BiCGStab (van der Vorst) with the two-level
-// Schwarz preconditioner (the element patches above and the coarse space below).  Its
-// scalars stay on the device: every dot product is reduced in two fixed stages (per-block
-// partial sums, then each reader sums the kKB partials in the same order), so the iteration
-// is deterministic and no kernel waits on the host; the host reads the convergence state
-// once every kCheck iterations.  One iteration is 11 launches: p; p_hat = M^{-1} p (element
-// patches with the coarse restriction, coarse solve, per-multiplier gather); v = H p_hat
-// with r_hat.v; s; s_hat (the same three); t = H s_hat with t.s and t.t; lambda and r with
-// r_hat.r and r.r.  The
-// kernels take their iteration as an offset from a base index held on the device, so one
-// CUDA graph of kCheck iterations (and the base's advance) is replayed block after block.
-constexpr int kKB = 256, kKT = 256, kCheck = 16;
-enum { kDotRV = 0, kDotTS = 1, kDotTT = 2, kDotRR_hat = 3, kDotRR = 4, kNumDots = 5 };
+// Schwarz preconditioner (the element patches above and the coarse space below) as one
+// cooperative kernel, kry_solve_kernel.  The mesh is cut into tiles of whole elements, each
+// inside one coarse cell; a CTA takes a tile (or several) and owns the multipliers of the
+// left and bottom faces of its elements.  Vectors that other tiles read live in global
+// memory and are read past L1; a phase's own intermediate (the vector the element patches or
+// the matrix act on, with its halo) sits in shared memory.  One iteration is four phases,
+// each closed by a grid barrier:
+//   A  omega, rho and beta from the last phase's dots; lambda, r and p of the owned
+//      multipliers; z_e = Pinv_e p|e per element; the cell's restriction of p; r.r
+//   B  p_hat = the two sides' z + the coarse correction, on the tile and
+//      its halo; v = H p_hat; r_hat.v
+//   C  convergence test on r.r; alpha; s = r - alpha v; z_e = Pinv_e s|e; restriction of s; r_hat.s
+//   D  s_hat as in B; t = H s_hat; t.s, t.t, r_hat.t
+// (rho of the next iteration is r_hat.s - omega r_hat.t, so it needs no barrier of its own).
+// Every dot product is summed in a fixed order (per tile, then over the tiles), so the
+// iteration is deterministic.  The waits at the barriers are bounded.
+constexpr int kKT = 512, kCheck = 256;   // threads per CTA; iterations per launch
+enum { kDotRR = 0, kDotRV = 1, kDotRS = 2, kDotTS = 3, kDotTT = 4, kDotRT = 5, kNumDots = 6 };
+constexpr size_t kTileSmemMax = 160 * 1024;
+constexpr unsigned kGridPolls = 1u << 22;   // a poll takes ~0.3 us or more: a second or so
 
-struct KScal { double rho, alpha, omega; };
 struct KState {
   int done;      // 1: converged, 2: breakdown
   int iters;     // iterations completed when done was set
-  int base;      // iterations launched before the current block
-  int pad;
+  int base;      // iterations completed by earlier launches
+  unsigned bar;  // arrivals at the grid barrier of the running launch
   double bb;     // ||r0||^2
   double rr;     // ||r||^2 at the last check
   double tol2;   // squared relative tolerance
+  double rho, alpha;   // of the last completed iteration
 };
 static_assert(sizeof(KState) % sizeof(double) == 0, "KState is carved from a double buffer");
 
@@ -820,89 +811,23 @@ struct Kry {
   // coarse space of the preconditioner: bilinear functions on a grid of (ncx+1) x (ncy+1)
   // vertices whose cells hold cx x cy elements (the last ones fewer)
   int ncx, ncy, cx, cy, nc;
+  // tiles: each cell cut into sx x sy sub-blocks of tw x th elements (the last ones fewer)
+  int sx, sy, tw, th, ntiles;
   double gl[kMaxP + 1];   // the multiplier nodes on [0, 1]
-  int* cv;                // [nl] lower-left coarse vertex of each multiplier's coarse cell
-  double2* cw;            // [nl] its local coordinates (xi, eta) in that cell
+  double2* cw;            // [nl] each multiplier's local coordinates (xi, eta) in its coarse cell
   double* A0;             // [nc][nc] the coarse operator R0 H R0^T, then its inverse
-  double* pc;             // [ncx ncy][4] per cell: its multipliers' restriction to its vertices
-  double* zc;             // [nc] coarse correction
-  double *x, *r, *rh, *p, *v, *s, *t, *ph, *sh;
-  double* part;   // [kNumDots][kKB]
-  KScal* sc;      // [iterations + 1]: sc[i] holds iteration i's rho, alpha, omega (sc[0] = 1)
+  double* pc;             // [ntiles][4] per tile: its multipliers' restriction to its cell's vertices
+  double *x, *r, *rh, *p[2], *v, *s, *t, *ph, *sh;
+  double* part;   // [kNumDots][ntiles]
   KState* st;
 };
-
-// whether an earlier launch ended the iteration (read once per block, so the whole block
-// leaves together)
-__device__ __forceinline__ bool kry_stopped(const Kry& k) {
-  __shared__ int done;
-  if (threadIdx.x == 0) done = *(volatile const int*)&k.st->done;
-  __syncthreads();
-  return done != 0;
-}
-
-// sum of the kKB partials of dot q, in a fixed order, broadcast to the block
-__device__ double kry_sum(const double* __restrict__ part, int q, double* red) {
-  if (threadIdx.x < 32) {
-    double a = 0.0;
-#pragma unroll
-    for (int i = 0; i < kKB / 32; ++i) a += part[q * kKB + threadIdx.x + 32 * i];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
-    if (threadIdx.x == 0) *red = a;
-  }
-  __syncthreads();
-  const double v = *red;
-  __syncthreads();
-  return v;
-}
-
-// block sums of a and b into part[qa][blockIdx], part[qb][blockIdx] (qb < 0: a only)
-__device__ void kry_partial(double a, double b, double* part, int qa, int qb) {
-  __shared__ double ra[kKT / 32], rb[kKT / 32];
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    a += __shfl_xor_sync(0xffffffffu, a, o);
-    b += __shfl_xor_sync(0xffffffffu, b, o);
-  }
-  const int w = threadIdx.x >> 5;
-  if ((threadIdx.x & 31) == 0) { ra[w] = a; rb[w] = b; }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double sa = 0.0, sb = 0.0;
-    for (int i = 0; i < (int)(blockDim.x >> 5); ++i) { sa += ra[i]; sb += rb[i]; }
-    part[qa * kKB + blockIdx.x] = sa;
-    if (qb >= 0) part[qb * kKB + blockIdx.x] = sb;
-  }
-}
-
-// The preconditioner's element half: z_e = Pinv_e x|e for every element and row (the face
-// half, each face's two sides summed, is kry_precond_gather_kernel), on blocks b of nb
-template <int P>
-__device__ __forceinline__ void asm_apply_blocks(const Kry& k, const double* __restrict__ x, unsigned b,
-                                                 unsigned nb) {
-  constexpr int NL = P + 1, NL4 = 4 * NL;
-  for (long long t = b * (long long)blockDim.x + threadIdx.x; t < k.E * NL4; t += (long long)nb * blockDim.x) {
-    const long long e = t / NL4;
-    const double* row = k.Pinv + (size_t)t * NL4;
-    double s = 0.0;
-#pragma unroll
-    for (int g = 0; g < 4; ++g) {
-      const long long fi = face_index(k.nx, k.ny, (int)e, g);
-      if (fi < 0) continue;
-#pragma unroll
-      for (int u = 0; u < NL; ++u) s = fma(row[g * NL + u], x[fi * NL + u], s);
-    }
-    k.z[t] = s;
-  }
-}
 
 // ---- coarse space of the preconditioner (two-level additive Schwarz): the coarse
 // functions are bilinear on a grid of at most 12 x 12 vertices laid over the elements, taken
 // at the multiplier nodes of every interior face; the coarse operator A0 = R0 H R0^T is
 // assembled from the elements' H_e and inverted once per solve, and each application adds
 // R0^T A0^{-1} R0 x to the element-patch part.
-// (144 vertices: the coarse operator, 162 KB in FP64, is inverted in one CTA's shared memory)
+// (144 vertices: the coarse operator is inverted in one CTA's shared memory)
 constexpr int kCoarseMaxCells = 11, kCoarseMax = (kCoarseMaxCells + 1) * (kCoarseMaxCells + 1);
 
 // the coarse cell holding multiplier node tt of interior face fid (its lower-left vertex v0)
@@ -959,7 +884,6 @@ __global__ void hrt_coarse_nodes_kernel(Kry k) {
   int v0;
   double xi, eta;
   coarse_coords(k, t / NL, (int)(t % NL), v0, xi, eta);
-  k.cv[t] = v0;
   k.cw[t] = make_double2(xi, eta);
 }
 
@@ -1053,11 +977,94 @@ __global__ void hrt_coarse_assemble_kernel(Kry k, const double* __restrict__ Ace
   if (mx == 0.0) row[a] = 1.0;
 }
 
-// Gauss-Jordan inverse of the coarse operator with partial pivoting, in FP32 in one CTA's
-// shared memory, of A0 scaled by its largest entry; written back in FP64 over A0.  The
-// coarse solve is part of the preconditioner only: its accuracy changes the iteration
-// count, not the FP64 Krylov iteration's answer.  (FP64 here is held to one SM's two FP64
-// FMA per clock: n^3 = 3 M FMA is 0.75 ms, FP32 runs at 64 times that rate.)
+// Gauss-Jordan inverse of the coarse operator, in FP32 in one CTA, of A0 scaled by its
+// largest entry; written back in FP64 over A0.  The coarse solve is part of the
+// preconditioner only: its accuracy changes the iteration count, not the FP64 Krylov
+// iteration's answer.  (FP64 here is held to one SM's two FP64 FMA per clock: n^3 = 3 M FMA
+// is 0.75 ms, FP32 runs at 64 times that rate.)  A0 is close to symmetric positive definite
+// (it is for E = I/3), so the elimination takes the diagonal pivots in order: 1024 threads
+// hold the matrix in registers, entry (i, j) on warp i mod 32, lane j mod 32, and a step
+// publishes the pivot row and column through a double buffer in shared memory, one barrier
+// and at most 25 FMA per thread.  A pivot below 2^-14 of its row's largest entry, or not
+// finite, leaves A0 as it is and raises *fallback, and hrt_coarse_pivot_kernel inverts it with
+// partial pivoting instead.
+constexpr int kCoarseTile = (kCoarseMax + 31) / 32;
+__global__ void __launch_bounds__(1024) hrt_coarse_invert_kernel(Kry k, int* __restrict__ fallback) {
+  const int n = k.nc, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  __shared__ float srow[2][32 * kCoarseTile], scol[2][32 * kCoarseTile];
+  __shared__ double wmax[32];
+  float a[kCoarseTile][kCoarseTile], scale[kCoarseTile];
+  double m = 0.0;
+  for (int idx = threadIdx.x; idx < n * n; idx += 1024) m = fmax(m, fabs(k.A0[idx]));
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+  if (lane == 0) wmax[warp] = m;
+  __syncthreads();
+  m = wmax[lane];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+  const double rs = m > 0.0 ? 1.0 / m : 1.0;
+#pragma unroll
+  for (int u = 0; u < kCoarseTile; ++u) {
+    float mx = 0.0f;
+#pragma unroll
+    for (int v = 0; v < kCoarseTile; ++v) {
+      const int i = warp + 32 * u, j = lane + 32 * v;
+      a[u][v] = i < n && j < n ? (float)(k.A0[i * n + j] * rs) : 0.0f;
+      mx = fmaxf(mx, fabsf(a[u][v]));
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    scale[u] = mx;
+  }
+  bool bad = false;
+#pragma unroll
+  for (int u0 = 0; u0 < kCoarseTile; ++u0) {
+    for (int kk = 0; kk < 32; ++kk) {
+      const int step = 32 * u0 + kk, b = step & 1;
+      if (step >= n) break;
+      if (warp == kk) {
+#pragma unroll
+        for (int v = 0; v < kCoarseTile; ++v) srow[b][lane + 32 * v] = a[u0][v];
+      }
+      if (lane == kk) {
+#pragma unroll
+        for (int u = 0; u < kCoarseTile; ++u) scol[b][warp + 32 * u] = a[u][u0];
+      }
+      __syncthreads();
+      const float piv = srow[b][step], inv = 1.0f / piv;
+      if (warp == kk) bad = bad || !(fabsf(piv) > scale[u0] * 6.103515625e-05f) || !isfinite(inv);
+      float r[kCoarseTile];
+#pragma unroll
+      for (int v = 0; v < kCoarseTile; ++v) r[v] = srow[b][lane + 32 * v] * inv;
+#pragma unroll
+      for (int u = 0; u < kCoarseTile; ++u) {
+        const float c = scol[b][warp + 32 * u];
+#pragma unroll
+        for (int v = 0; v < kCoarseTile; ++v) a[u][v] = fmaf(-c, r[v], a[u][v]);
+        if (lane == kk) a[u][u0] = -c * inv;
+      }
+      if (warp == kk) {
+#pragma unroll
+        for (int v = 0; v < kCoarseTile; ++v) a[u0][v] = r[v];
+        if (lane == kk) a[u0][u0] = inv;
+      }
+    }
+  }
+  const bool any = __syncthreads_or(bad) != 0;
+  if (threadIdx.x == 0) *fallback = any;
+  if (any) return;
+#pragma unroll
+  for (int u = 0; u < kCoarseTile; ++u)
+#pragma unroll
+    for (int v = 0; v < kCoarseTile; ++v) {
+      const int i = warp + 32 * u, j = lane + 32 * v;
+      if (i < n && j < n) k.A0[i * n + j] = (double)a[u][v] * rs;
+    }
+}
+
+// The same inverse with partial pivoting, for an A0 whose diagonal pivots were too small (the
+// kernel leaves at once otherwise).
 // Per pivot step two barriers: every warp finds the pivot row itself (same order, same
 // result), the pivot row, the row it changes places with and the pivot column go to
 // buffers, and each thread then updates only its own entries, reading the row that moves
@@ -1065,7 +1072,9 @@ __global__ void hrt_coarse_assemble_kernel(Kry k, const double* __restrict__ Ace
 // FP32) drops the coarse part: the inverse is written as zero and the preconditioner is the
 // element patches alone.
 constexpr int kCoarseInvThreads = 512, kCoarsePerLane = (kCoarseMax + 31) / 32;
-__global__ void __launch_bounds__(kCoarseInvThreads) hrt_coarse_invert_kernel(Kry k) {
+__global__ void __launch_bounds__(kCoarseInvThreads)
+hrt_coarse_pivot_kernel(Kry k, const int* __restrict__ fallback) {
+  if (*fallback == 0) return;
   const int n = k.nc, ld = n | 1, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   constexpr int nwarp = kCoarseInvThreads / 32;
   extern __shared__ float A[];   // [n][ld]
@@ -1146,268 +1155,560 @@ __global__ void __launch_bounds__(kCoarseInvThreads) hrt_coarse_invert_kernel(Kr
   }
 }
 
-// per coarse cell (one CTA): the restriction of x to its four vertices from the multiplier
-// nodes the cell owns (coarse_coords), threads in a fixed stride and a fixed-order block sum
+// element ranges of tile q: its cell (kx, ky) and [i0, i1) x [j0, j1) (empty for a sub-block
+// past a short cell's end); r1, r2: multipliers for division by the width + 1, + 2
+struct KTile { int kx, ky, i0, i1, j0, j1; unsigned r0, r1, r2; };
+__device__ __forceinline__ KTile kry_tile(const Kry& k, int q) {
+  const int ns = k.sx * k.sy, cell = q / ns, sub = q - cell * ns;
+  KTile t;
+  t.kx = cell % k.ncx;
+  t.ky = cell / k.ncx;
+  const int ie = min((t.kx + 1) * k.cx, k.nx), je = min((t.ky + 1) * k.cy, k.ny);
+  t.i0 = min(t.kx * k.cx + (sub % k.sx) * k.tw, ie);
+  t.j0 = min(t.ky * k.cy + (sub / k.sx) * k.th, je);
+  t.i1 = min(t.i0 + k.tw, ie);
+  t.j1 = min(t.j0 + k.th, je);
+  const unsigned w = (unsigned)(t.i1 - t.i0);
+  t.r0 = w > 1 ? 0xffffffffu / w + 1 : 0;
+  t.r1 = w > 0 ? 0xffffffffu / (w + 1) + 1 : 0;
+  t.r2 = 0xffffffffu / (w + 2) + 1;
+  return t;
+}
+// a / d by the multiplier r = 2^32 / d rounded up (0 stands for d = 1): exact for the element
+// counts of a tile (a d < 2^32)
+__device__ __forceinline__ int kry_div(int a, unsigned r) { return r ? (int)__umulhi((unsigned)a, r) : a; }
+// multiplier of node tt on the left (side 0) or bottom face of element (i, j)
 template <int P>
-__device__ __forceinline__ void coarse_restrict_cell(const Kry& k, const double* __restrict__ x, int cell) {
-  constexpr int NL = P + 1;
-  const int kx = cell % k.ncx, ky = cell / k.ncx;
-  const int i0 = kx * k.cx, i1 = min(i0 + k.cx, k.nx), j0 = ky * k.cy, j1 = min(j0 + k.cy, k.ny);
-  const long long nv = (long long)(k.nx - 1) * k.ny;
-  const int xa = max(i0, 1), ya = max(j0, 1);
-  const int nvf = max(0, i1 - xa) * (j1 - j0), nhf = max(0, j1 - ya) * (i1 - i0);
-  double acc[4] = {0.0, 0.0, 0.0, 0.0};
-  for (int t = threadIdx.x; t < (nvf + nhf) * NL; t += blockDim.x) {
-    const int fl = t / NL, tt = t - fl * NL;
-    long long fid;
-    if (fl < nvf) {
-      const int xv = xa + fl / (j1 - j0), j = j0 + fl % (j1 - j0);
-      fid = (long long)j * (k.nx - 1) + (xv - 1);
-    } else {
-      const int g = fl - nvf, yh = ya + g / (i1 - i0), i = i0 + g % (i1 - i0);
-      fid = nv + (long long)(yh - 1) * k.nx + i;
+__device__ __forceinline__ int kry_dof(const Kry& k, int side, int i, int j, int tt) {
+  return (side == 0 ? j * (k.nx - 1) + i - 1 : (k.nx - 1) * k.ny + (j - 1) * k.nx + i) * (P + 1) + tt;
+}
+
+// Grid barrier of a cooperative launch (all CTAs resident): arrivals are counted up from zero
+// over the launch.  Bounded: when the polls run out the timeout bit is set and every CTA that
+// sees the count short leaves.  Returns whether the barrier completed.
+__device__ __forceinline__ bool kry_barrier(KState* st, unsigned& epoch, unsigned int* status) {
+  __shared__ int ok;
+  epoch += gridDim.x;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    atomicAdd(&st->bar, 1u);
+    unsigned n = 0;
+    while ((unsigned)ld_acquire_gpu((const int*)&st->bar) < epoch && ++n < kGridPolls) {
     }
-    const long long q = fid * NL + tt;
-    const double2 c = k.cw[q];
-    double w[4];
-    bilinear(c.x, c.y, w);
-    const double xq = x[q];
-#pragma unroll
-    for (int b = 0; b < 4; ++b) acc[b] = fma(w[b], xq, acc[b]);
-  }
-  __shared__ double red[8][4];
-#pragma unroll
-  for (int b = 0; b < 4; ++b) {
-    double v = acc[b];
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5][b] = v;
+    ok = n < kGridPolls;
+    if (n >= kGridPolls) atomicOr(status, kDevTimeout);
   }
   __syncthreads();
-  if (threadIdx.x < 4) {
-    double sum = 0.0;
-    for (int i = 0; i < (int)(blockDim.x >> 5); ++i) sum += red[i][threadIdx.x];
-    k.pc[(size_t)cell * 4 + threadIdx.x] = sum;
-  }
+  return ok != 0;
 }
 
-// the two parts of an application that read only x, in one launch: blocks [0, napply) the
-// element patches, the rest one coarse cell each
-template <int P>
-__global__ void __launch_bounds__(256) kry_precond_local_kernel(Kry k, const double* __restrict__ x,
-                                                                unsigned napply) {
-  if (kry_stopped(k)) return;
-  if (blockIdx.x < napply) asm_apply_blocks<P>(k, x, blockIdx.x, napply);
-  else coarse_restrict_cell<P>(k, x, (int)(blockIdx.x - napply));
+// The scalars of the iteration, kept by thread 0 of every CTA (the same values in the same
+// order everywhere) and read by the others from shared memory: an FP64 division or comparison
+// costs its warp's sub-partition as much as a multiply-add, and 16 warps repeating it cost 16
+// times that.
+struct KryScal {
+  double dot[4];
+  double rho, rho_new, alpha, omega, beta, bb, rr, tol2;
+  int it, done, iters, brk;
+};
+
+// a / b to within two ulp: the approximate reciprocal refined by two Newton-Raphson steps
+// (pivot_rcp), at a third of a division's dependent FP64 operations; an operand outside the
+// reciprocal's range divides
+__device__ __forceinline__ double kry_quot(double a, double b) {
+  const double q = a * pivot_rcp(b);
+  return isfinite(q) ? q : a / b;
 }
 
-// zc = A0^{-1} vc, vc summed per vertex from the cells around it (fixed order) into shared
-// memory by every block, then one warp per row
-__global__ void __launch_bounds__(256) kry_coarse_solve_kernel(Kry k) {
-  if (kry_stopped(k)) return;
-  __shared__ double vc[kCoarseMax];
-  const int W = k.ncx + 1;
-  for (int a = threadIdx.x; a < k.nc; a += blockDim.x) {
-    const int ax = a % W, ay = a / W;
-    double v = 0.0;
-    for (int cy = ay - 1; cy <= ay; ++cy)
-      for (int cx = ax - 1; cx <= ax; ++cx) {
-        if (cx < 0 || cy < 0 || cx >= k.ncx || cy >= k.ncy) continue;
-        v += k.pc[(size_t)(cy * k.ncx + cx) * 4 + (ay - cy) * 2 + (ax - cx)];
-      }
-    vc[a] = v;
+// the sums over the tiles of nq <= 4 dots q, warp w summing dot q[w] in a fixed order, into
+// sc.dot; ends with a block barrier
+__device__ __forceinline__ void kry_sums(const Kry& k, KryScal& sc, int q0, int q1, int q2, int q3, int nq) {
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (w < nq) {
+    const double* p = k.part + (size_t)(w == 0 ? q0 : w == 1 ? q1 : w == 2 ? q2 : q3) * k.ntiles;
+    double a = 0.0;
+    for (int i = lane; i < k.ntiles; i += 32) a += __ldcg(p + i);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+    if (lane == 0) sc.dot[w] = a;
   }
   __syncthreads();
-  const int row = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-  if (row >= k.nc) return;
-  const double* Ar = k.A0 + (size_t)row * k.nc;
-  double s = 0.0;
-  for (int b = lane; b < k.nc; b += 32) s = fma(Ar[b], vc[b], s);
-  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  if (lane == 0) k.zc[row] = s;
 }
 
-// y = M^{-1} x assembled per multiplier: the two sides' element-patch results plus the
-// coarse correction R0^T zc
+// K values per lane (a power of two) summed over the warp in log2(K) halving exchanges and a
+// butterfly of one value: K - 1 + 5 - log2(K) additions instead of 5 K.  Lane l ends with the
+// total of value kry_which<K>(l) in v[0].
+template <int K>
+__device__ __forceinline__ void kry_warp_sums(double (&v)[K]) {
+  const int lane = threadIdx.x & 31;
+  int off = 16;
+#pragma unroll
+  for (int h = K / 2; h >= 1; h >>= 1) {
+    const bool up = (lane & off) != 0;
+#pragma unroll
+    for (int i = 0; i < h; ++i) {
+      const double send = up ? v[i] : v[i + h], keep = up ? v[i + h] : v[i];
+      v[i] = keep + __shfl_xor_sync(0xffffffffu, send, off);
+    }
+    off >>= 1;
+  }
+#pragma unroll
+  for (; off > 0; off >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], off);
+}
+template <int K>
+__device__ __forceinline__ int kry_which(int lane) {
+  int idx = 0;
+  for (int h = K / 2, bit = 4; h >= 1; h >>= 1, --bit) idx += ((lane >> bit) & 1) * h;
+  return idx;
+}
+
+// block sums of NV <= K values per thread in a fixed order; store(i, total) is called once per
+// value.  Only the warps that had one of the `items` work items add (16 idle warps' shuffled
+// additions would cost a microsecond).  Ends with a block barrier.
+template <int NV, int K, typename F>
+__device__ __forceinline__ void kry_block_sums(double (&val)[K], int items, F store) {
+  __shared__ double red[K][kKT / 32];
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int nw = min(kKT / 32, max(1, (items + 31) / 32));
+  if (w < nw) {
+    kry_warp_sums<K>(val);
+    if ((lane & (32 / K - 1)) == 0) red[kry_which<K>(lane)][w] = val[0];
+  }
+  __syncthreads();
+  if (w < NV) {
+    double a = lane < nw ? red[w][lane] : 0.0;
+    for (int o = nw > 4 ? kKT / 64 : nw > 1 ? 2 : 0; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+    if (lane == 0) store(w, a);
+  }
+  __syncthreads();
+}
+
+// one row of an element matrix (H_e or Pinv_e) times the element's multipliers, staged at x0 of a buffer W elements
+// wide (faces in order bottom, right = the next element's left, top = the upper one's bottom,
+// left)
 template <int P>
-__global__ void kry_precond_gather_kernel(Kry k, double* __restrict__ y) {
+__device__ __forceinline__ double kry_row(const double* __restrict__ M, int e, int row,
+                                          const double* __restrict__ x0, int W) {
   constexpr int NL = P + 1, NL4 = 4 * NL;
-  const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (t >= k.nl) return;
-  long long e1, e2;
-  int f1, f2;
-  face_sides(k.nx, k.ny, t / NL, e1, f1, e2, f2);
-  const int tt = (int)(t % NL);
-  const int v0 = k.cv[t], W = k.ncx + 1;
-  const double2 c = k.cw[t];
-  double w[4];
-  bilinear(c.x, c.y, w);
-  const double cor = fma(w[3], k.zc[v0 + W + 1], fma(w[2], k.zc[v0 + W], fma(w[1], k.zc[v0 + 1], w[0] * k.zc[v0])));
-  y[t] = (k.z[e1 * NL4 + f1 * NL + tt] + k.z[e2 * NL4 + f2 * NL + tt]) + cor;
+  const double2* A = reinterpret_cast<const double2*>(M + (size_t)(e * NL4 + row) * NL4);
+  const double* xf[4] = {x0 + NL, x0 + 2 * NL, x0 + (size_t)W * 2 * NL + NL, x0};
+  double s = 0.0;
+#pragma unroll
+  for (int h = 0; h < NL4 / 2; ++h) {
+    const double2 a = __ldg(A + h);
+    s = fma(a.x, xf[(2 * h) / NL][(2 * h) % NL], s);
+    s = fma(a.y, xf[(2 * h + 1) / NL][(2 * h + 1) % NL], s);
+  }
+  return s;
 }
 
-// r_hat = r, x = p = v = 0, partials of r_hat.r and r.r, sc[0] = 1, state cleared
-__global__ void kry_init_kernel(Kry k, double tol2) {
-  double a = 0.0;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < k.nl; i += (long long)gridDim.x * blockDim.x) {
-    const double ri = k.r[i];
-    k.rh[i] = ri;
-    k.x[i] = 0.0; k.p[i] = 0.0; k.v[i] = 0.0;
-    a = fma(ri, ri, a);
-  }
-  kry_partial(a, a, k.part, kDotRR_hat, kDotRR);
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    k.sc[0] = KScal{1.0, 1.0, 1.0};
-    *k.st = KState{0, 0, 0, 0, 0.0, 0.0, tol2};
-  }
-}
-
-// iteration base + j, step 1: convergence test on the previous residual, rho, p.
-// With update == false it only records the state (the final check after the last
-// iteration).
+// z_e = Pinv_e x|e for the tile's elements, x staged in sx as [element of the tile widened by
+// one column and row][left, bottom][node]
 template <int P>
-__global__ void kry_p_kernel(Kry k, int j, bool update) {
-  __shared__ double red;
-  if (kry_stopped(k)) return;
-  const int it = k.st->base + j;
-  const double rr = kry_sum(k.part, kDotRR, &red);
-  const double rho = kry_sum(k.part, kDotRR_hat, &red);
-  const double bb = it == 0 ? rr : k.st->bb;
-  const bool conv = rr <= k.st->tol2 * bb;
-  const KScal pv = k.sc[it];
-  const bool brk = !conv && update && (rho == 0.0 || !isfinite(rho) || pv.omega == 0.0);
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    if (it == 0) k.st->bb = rr;
-    k.st->rr = rr;
-    if (conv || brk) { k.st->done = conv ? 1 : 2; k.st->iters = it; }
-    k.sc[it + 1].rho = rho;
+__device__ __forceinline__ void kry_patches(const Kry& k, const KTile& t, const double* __restrict__ sx) {
+  constexpr int NL = P + 1, NL4 = 4 * NL;
+  const int w = t.i1 - t.i0, nel = w * (t.j1 - t.j0), W = w + 1;
+  for (int q = threadIdx.x; q < nel * NL4; q += kKT) {
+    const int le = q / NL4, row = q - le * NL4, lj = kry_div(le, t.r0), li = le - lj * w;
+    const int e = (t.j0 + lj) * k.nx + t.i0 + li;
+    k.z[e * NL4 + row] = kry_row<P>(k.Pinv, e, row, sx + (size_t)(lj * W + li) * 2 * NL, W);
   }
-  if (conv || brk || !update) return;
-  const double beta = (rho / pv.rho) * (pv.alpha / pv.omega);
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < k.nl; i += (long long)gridDim.x * blockDim.x)
-    k.p[i] = k.r[i] + beta * (k.p[i] - pv.omega * k.v[i]);
 }
 
-// y = H x with the partial dots w.y (into qa) and, when qb >= 0, y.y (into qb)
-template <int P>
-__global__ void kry_matvec_kernel(Kry k, const double* __restrict__ x, double* __restrict__ y,
-                                  const double* __restrict__ w, int qa, int qb) {
-  constexpr int NL = P + 1;
-  if (kry_stopped(k)) return;
-  double a = 0.0, b = 0.0;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < k.nl; i += (long long)gridDim.x * blockDim.x) {
-    long long e1, e2;
-    int f1, f2;
-    face_sides(k.nx, k.ny, i / NL, e1, f1, e2, f2);
-    const int tt = (int)(i % NL);
-    const double yi = he_row<P>(k.nx, k.ny, k.He, x, e1, f1, tt) + he_row<P>(k.nx, k.ny, k.He, x, e2, f2, tt);
-    y[i] = yi;
-    a = fma(w[i], yi, a);
-    b = fma(yi, yi, b);
+// The coarse correction around the tile's cell: every CTA sums the restriction per vertex
+// from the cells around it (fixed order), multiplies the rows of A0^{-1} it needs and forms
+// each of the 3 x 3 cells' bilinear coefficients: correction = c0 + c1 xi + (c2 + c3 xi) eta.
+// The matrix needs the correction on the tile, on the faces of the elements to its left and
+// below, and on the left / bottom faces of the next column / row, which lie on that cell's
+// line (xi = 0 / eta = 0): vertices (kx - 1 .. kx + 1) x (ky - 1 .. ky + 1); the vertices
+// beyond are taken as zero.  A tile's restriction comes as
+// the sums of x, xi x, eta x and xi eta x over its multipliers.
+__device__ __forceinline__ void kry_coarse(const Kry& k, const double (*a0)[kCoarseMax], double* vc, double* zc,
+                                           double (*cc)[4]) {
+  const int W = k.ncx + 1, ns = k.sx * k.sy;
+  for (int a = threadIdx.x; a < k.nc; a += kKT) {
+    const int ay = a / W, ax = a - ay * W;
+    // the vertex is cell c's upper right (c = 0), upper left, lower right, lower left corner
+    double q[4];
+    if (ns == 1) {   // the cells' values read together
+      double2 s01[4], s23[4];
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        const int cx = ax - 1 + (c & 1), cy = ay - 1 + (c >> 1);
+        const bool in = cx >= 0 && cy >= 0 && cx < k.ncx && cy < k.ncy;
+        const double2* p = reinterpret_cast<const double2*>(k.pc) + (in ? cy * k.ncx + cx : 0) * 2;
+        s01[c] = in ? __ldcg(p) : make_double2(0.0, 0.0);
+        s23[c] = in ? __ldcg(p + 1) : make_double2(0.0, 0.0);
+      }
+      q[0] = s23[0].y;
+      q[1] = s23[1].x - s23[1].y;
+      q[2] = s01[2].y - s23[2].y;
+      q[3] = (s01[3].x - s01[3].y) - (s23[3].x - s23[3].y);
+    } else {
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        const int cx = ax - 1 + (c & 1), cy = ay - 1 + (c >> 1);
+        double v = 0.0;
+        if (cx >= 0 && cy >= 0 && cx < k.ncx && cy < k.ncy) {
+          const double2* p = reinterpret_cast<const double2*>(k.pc) + (size_t)(cy * k.ncx + cx) * ns * 2;
+          for (int u = 0; u < ns; ++u) {
+            const double2 s01 = __ldcg(p + 2 * u), s23 = __ldcg(p + 2 * u + 1);
+            v += c == 0 ? s23.y : c == 1 ? s23.x - s23.y : c == 2 ? s01.y - s23.y : (s01.x - s01.y) - (s23.x - s23.y);
+          }
+        }
+        q[c] = v;
+      }
+    }
+    vc[a] = (q[0] + q[1]) + (q[2] + q[3]);
   }
-  kry_partial(a, b, k.part, qa, qb);
+  __syncthreads();
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (w < 4) {   // warp w: the three vertices of row ky - 1 + w
+    double s[4] = {0.0, 0.0, 0.0, 0.0};
+    if (w < 3) {
+      for (int b = lane; b < k.nc; b += 32) {
+        const double vb = vc[b];
+#pragma unroll
+        for (int i = 0; i < 3; ++i) s[i] = fma(a0[3 * w + i][b], vb, s[i]);
+      }
+      kry_warp_sums<4>(s);
+    }
+    if ((lane & 7) == 0) zc[4 * w + kry_which<4>(lane)] = s[0];
+  }
+  __syncthreads();
+  if (threadIdx.x < 9) {
+    const double* z = zc + (threadIdx.x / 3) * 4 + threadIdx.x % 3;
+    double* c = cc[threadIdx.x];
+    c[0] = z[0];
+    c[1] = z[1] - z[0];
+    c[2] = z[4] - z[0];
+    c[3] = (z[5] - z[4]) - (z[1] - z[0]);
+  }
+  __syncthreads();
+}
+// the rows of A0^{-1} of the vertices (kx - 1 .. kx + 1) x (ky - 1 .. ky + 1) into shared memory
+__device__ __forceinline__ void kry_load_rows(const Kry& k, const KTile& t, double (*a0)[kCoarseMax]) {
+  for (int i = threadIdx.x; i < 9 * k.nc; i += kKT) {
+    const int r = i / k.nc, b = i - r * k.nc, ax = t.kx - 1 + r % 3, ay = t.ky - 1 + r / 3;
+    a0[r][b] = ax >= 0 && ay >= 0 ? k.A0[(size_t)(ay * (k.ncx + 1) + ax) * k.nc + b] : 0.0;
+  }
+  __syncthreads();
 }
 
-// step 3: alpha, s = r - alpha v
+// y = M^{-1} x on the tile and one element around it: the two sides' element-patch results
+// plus the coarse correction, into sy as [element of the widened tile][left, bottom][node]
+// (zero on boundary faces); the owned values also to out
 template <int P>
-__global__ void kry_s_kernel(Kry k, int j) {
-  __shared__ double red;
-  if (kry_stopped(k)) return;
-  const int it = k.st->base + j;
-  const double rv = kry_sum(k.part, kDotRV, &red);
-  const double alpha = k.sc[it + 1].rho / rv;
-  if (!isfinite(alpha)) {
-    if (blockIdx.x == 0 && threadIdx.x == 0) { k.st->done = 2; k.st->iters = it; }
+__device__ __forceinline__ void kry_gather(const Kry& k, const KTile& t, const double (*cc)[4], double* sy,
+                                           double* __restrict__ out) {
+  constexpr int NL = P + 1, NL4 = 4 * NL;
+  const int W = t.i1 - t.i0 + 2, nel = W * (t.j1 - t.j0 + 2);
+  // the coarse cells' lines around the tile's cell
+  const int xl = t.kx * k.cx, xr = xl + k.cx, yl = t.ky * k.cy, yr = yl + k.cy;
+  for (int q = threadIdx.x; q < nel * 2 * NL; q += kKT) {
+    const int le = q / (2 * NL), c = q - le * 2 * NL, side = c / NL, tt = c - side * NL;
+    const int lj = kry_div(le, t.r2), i = t.i0 - 1 + le - lj * W, j = t.j0 - 1 + lj;
+    double y = 0.0;
+    if (i >= 0 && j >= 0 && i < k.nx && j < k.ny && (side == 0 ? i > 0 : j > 0)) {
+      const int e = j * k.nx + i, m = kry_dof<P>(k, side, i, j, tt);
+      const double z1 = __ldcg(k.z + (side == 0 ? (e - 1) * NL4 + NL : (e - k.nx) * NL4 + 2 * NL) + tt);
+      const double z2 = __ldcg(k.z + e * NL4 + (side == 0 ? 3 * NL : 0) + tt);
+      const double2 cw = k.cw[m];
+      // the face's cell is its element's
+      const double* d = cc[(j < yl ? 0 : j < yr ? 3 : 6) + (i < xl ? 0 : i < xr ? 1 : 2)];
+      y = fma(cw.y, fma(cw.x, d[3], d[2]), fma(cw.x, d[1], d[0] + (z1 + z2)));
+      if (i >= t.i0 && i < t.i1 && j >= t.j0 && j < t.j1) out[m] = y;
+    }
+    sy[q] = y;
+  }
+  __syncthreads();
+}
+
+// y = H x on the tile's owned multipliers (x staged by kry_gather); use(index, y) for each.
+// Large tiles: a lane per multiplier sums both sides' rows of H_e.  Small ones (at most kKT
+// items): two lanes per multiplier, one for each side's row, which keeps more sub-partitions at
+// work; the row, which does not depend on x, is fetched before x is formed (kry_fetch), so
+// that its latency overlaps the coarse solve and the gather.
+template <int P>
+__device__ __forceinline__ int kry_apply_items(const KTile& t) {
+  const int own = (t.i1 - t.i0) * (t.j1 - t.j0) * 2 * (P + 1);
+  return 2 * own <= kKT ? 2 * own : own;
+}
+template <int P>
+struct KFetch {
+  double2 a[2 * (P + 1)];
+  const double* x0;   // the row's element in the staged buffer
+  int m;              // the multiplier, or -1
+};
+template <int P>
+__device__ __forceinline__ void kry_fetch(const Kry& k, const KTile& t, const double* sy, KFetch<P>& r) {
+  constexpr int NL = P + 1, NL4 = 4 * NL;
+  const int w = t.i1 - t.i0, own = w * (t.j1 - t.j0) * 2 * NL, W = w + 2;
+  r.m = -1;
+  if (2 * own > kKT || (int)threadIdx.x >= 2 * own) return;
+  const int d = threadIdx.x >> 1, which = threadIdx.x & 1;
+  const int le = d / (2 * NL), c = d - le * 2 * NL, side = c / NL, tt = c - side * NL;
+  const int lj = kry_div(le, t.r0), li = le - lj * w, i = t.i0 + li, j = t.j0 + lj;
+  if (side == 0 ? i == 0 : j == 0) return;
+  // the element on the left / below (its right / top face), or the owner
+  const int di = which == 0 && side == 0, dj = which == 0 && side == 1;
+  const int e = (j - dj) * k.nx + i - di, row = (which == 0 ? (side == 0 ? NL : 2 * NL) : (side == 0 ? 3 * NL : 0)) + tt;
+  r.m = kry_dof<P>(k, side, i, j, tt);
+  r.x0 = sy + ((lj + 1 - dj) * W + li + 1 - di) * 2 * NL;
+  const double2* A = reinterpret_cast<const double2*>(k.He + (size_t)(e * NL4 + row) * NL4);
+#pragma unroll
+  for (int h = 0; h < NL4 / 2; ++h) r.a[h] = __ldg(A + h);
+}
+template <int P, typename F>
+__device__ __forceinline__ void kry_apply(const Kry& k, const KTile& t, const double* __restrict__ sy,
+                                          const KFetch<P>& r, F use) {
+  constexpr int NL = P + 1, NL4 = 4 * NL;
+  const int w = t.i1 - t.i0, own = w * (t.j1 - t.j0) * 2 * NL, W = w + 2;
+  if (2 * own <= kKT) {
+    double s = 0.0;
+    if (r.m >= 0) {
+      const double* x0 = r.x0;
+      const double* xf[4] = {x0 + NL, x0 + 2 * NL, x0 + W * 2 * NL + NL, x0};
+#pragma unroll
+      for (int h = 0; h < NL4 / 2; ++h) {
+        s = fma(r.a[h].x, xf[(2 * h) / NL][(2 * h) % NL], s);
+        s = fma(r.a[h].y, xf[(2 * h + 1) / NL][(2 * h + 1) % NL], s);
+      }
+    }
+    s += __shfl_xor_sync(0xffffffffu, s, 1);
+    if (r.m >= 0 && (threadIdx.x & 1)) use(r.m, s);
     return;
   }
-  if (blockIdx.x == 0 && threadIdx.x == 0) k.sc[it + 1].alpha = alpha;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < k.nl; i += (long long)gridDim.x * blockDim.x)
-    k.s[i] = k.r[i] - alpha * k.v[i];
-}
-
-// step 5: omega, lambda += alpha p_hat + omega s_hat, r = s - omega t, and the partials of
-// r_hat.r and r.r for the next iteration's test
-__global__ void kry_x_kernel(Kry k, int j) {
-  __shared__ double red;
-  if (kry_stopped(k)) return;
-  const int it = k.st->base + j;
-  const double ts = kry_sum(k.part, kDotTS, &red);
-  const double tt = kry_sum(k.part, kDotTT, &red);
-  const double alpha = k.sc[it + 1].alpha;
-  const double omega = tt > 0.0 ? ts / tt : 0.0;
-  if (blockIdx.x == 0 && threadIdx.x == 0) k.sc[it + 1].omega = omega;
-  double a = 0.0, b = 0.0;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < k.nl; i += (long long)gridDim.x * blockDim.x) {
-    k.x[i] += alpha * k.ph[i] + omega * k.sh[i];
-    const double ri = k.s[i] - omega * k.t[i];
-    k.r[i] = ri;
-    a = fma(k.rh[i], ri, a);
-    b = fma(ri, ri, b);
+  for (int q = threadIdx.x; q < own; q += kKT) {
+    const int le = q / (2 * NL), c = q - le * 2 * NL, side = c / NL, tt = c - side * NL;
+    const int lj = kry_div(le, t.r0), li = le - lj * w, i = t.i0 + li, j = t.j0 + lj;
+    if (side == 0 ? i == 0 : j == 0) continue;
+    const int e = j * k.nx + i;
+    const double* x0 = sy + ((lj + 1) * W + li + 1) * 2 * NL;
+    use(kry_dof<P>(k, side, i, j, tt),
+        side == 0 ? kry_row<P>(k.He, e - 1, NL + tt, x0 - 2 * NL, W) + kry_row<P>(k.He, e, 3 * NL + tt, x0, W)
+                  : kry_row<P>(k.He, e - k.nx, 2 * NL + tt, x0 - W * 2 * NL, W) + kry_row<P>(k.He, e, tt, x0, W));
   }
-  kry_partial(a, b, k.part, kDotRR_hat, kDotRR);
 }
 
-// the base index advances past a block of n iterations
-__global__ void kry_bump_kernel(KState* st, int n) { st->base += n; }
+template <int P>
+__device__ __forceinline__ int kry_stage_items(const KTile& t) {
+  return (t.i1 - t.i0 + 1) * (t.j1 - t.j0 + 1) * 2 * (P + 1);
+}
+// Stages x on the tile and one column and row to its right and top for kry_patches: value(m)
+// gives x at multiplier m, own(m, x, (xi, eta)) is called for the owned ones with their
+// local coordinates in the coarse cell.  Zero on boundary faces.
+template <int P, typename V, typename O>
+__device__ __forceinline__ void kry_stage(const Kry& k, const KTile& t, double* sx, V value, O own) {
+  constexpr int NL = P + 1;
+  const int W = t.i1 - t.i0 + 1, nel = W * (t.j1 - t.j0 + 1);
+  for (int q = threadIdx.x; q < nel * 2 * NL; q += kKT) {
+    const int le = q / (2 * NL), c = q - le * 2 * NL, side = c / NL, tt = c - side * NL;
+    const int lj = kry_div(le, t.r1), i = t.i0 + le - lj * W, j = t.j0 + lj;
+    double x = 0.0;
+    if (i < k.nx && j < k.ny && (side == 0 ? i > 0 : j > 0)) {
+      const int m = kry_dof<P>(k, side, i, j, tt);
+      x = value(m);
+      if (i < t.i1 && j < t.j1) own(m, x, k.cw[m]);
+    }
+    sx[q] = x;
+  }
+  __syncthreads();
+}
+
+// sums of x, xi x, eta x and xi eta x: a tile's restriction to its coarse cell
+__device__ __forceinline__ void kry_restrict(double (&acc)[8], double x, double2 c) {
+  const double tx = c.x * x;
+  acc[0] += x;
+  acc[1] += tx;
+  acc[2] = fma(c.y, x, acc[2]);
+  acc[3] = fma(c.y, tx, acc[3]);
+}
+
+// n iterations from the state left by the last launch (st->base of them done); check: then
+// the convergence test on the residual they leave.  Dynamic shared memory: the staged vector
+// of one tile with its halo.
+template <int P>
+__global__ void __launch_bounds__(kKT, 1) kry_solve_kernel(Kry k, int n, int check, unsigned int* status) {
+  extern __shared__ double sv[];
+  __shared__ double vc[kCoarseMax], zc[16], cc[9][4], a0[9][kCoarseMax];
+  __shared__ KryScal sc;
+  KState* st = k.st;
+  const bool lead = threadIdx.x == 0;
+  unsigned epoch = 0;
+  int it = st->base;
+  if (lead) {
+    sc.rho = st->rho;
+    sc.alpha = st->alpha;
+    sc.bb = st->bb;
+    sc.rr = st->rr;
+    sc.tol2 = st->tol2;
+    sc.done = st->done;
+    sc.iters = st->iters;
+  }
+  __syncthreads();
+  auto part = [&](int q, int tile) -> double& { return k.part[(size_t)q * k.ntiles + tile]; };
+  // usually one tile per CTA: its ranges and rows of A0^{-1} are kept
+  const KTile t0 = kry_tile(k, min((int)blockIdx.x, k.ntiles - 1));
+  const bool one = k.ntiles <= (int)gridDim.x;
+  kry_load_rows(k, t0, a0);
+  for (int j = 0; !sc.done; ++j) {
+    if (j == n && !check) break;
+    // ---- A
+    if (it > 0) {
+      kry_sums(k, sc, kDotTS, kDotTT, kDotRS, kDotRT, 4);
+      if (threadIdx.x < 32) {
+        // beta = (rho' / rho) (alpha / omega): its three divisions on three lanes at once
+        const int l = threadIdx.x;
+        const double q = kry_quot(l == 0 ? sc.dot[0] : l == 1 ? sc.dot[1] : sc.alpha,
+                                  l == 0 ? sc.dot[1] : l == 1 ? sc.dot[0] : sc.rho);
+        const double ti = __shfl_sync(0xffffffffu, q, 1), ar = __shfl_sync(0xffffffffu, q, 2);
+        if (lead) {
+          const double omega = sc.dot[1] > 0.0 ? q : 0.0;
+          const double rho = sc.dot[2] - omega * sc.dot[3];
+          const bool brk = rho == 0.0 || !isfinite(rho) || omega == 0.0;
+          sc.omega = omega;
+          sc.rho_new = rho;
+          sc.brk = brk;
+          sc.beta = brk ? 0.0 : rho * ar * ti;
+        }
+      }
+      __syncthreads();
+    }
+    const double omega = sc.omega, beta = sc.beta, alpha = sc.alpha;
+    const double* po = k.p[it & 1];
+    double* pn = k.p[(it & 1) ^ 1];
+    for (int tile = blockIdx.x; tile < k.ntiles; tile += gridDim.x) {
+      const KTile t = one ? t0 : kry_tile(k, tile);
+      double acc[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+      double ri = 0.0;   // r at the value just formed
+      kry_stage<P>(
+          k, t, sv,
+          [&](int m) {
+            if (it == 0) return ri = __ldcg(k.r + m);
+            ri = fma(-omega, __ldcg(k.t + m), __ldcg(k.s + m));
+            return fma(beta, fma(-omega, __ldcg(k.v + m), __ldcg(po + m)), ri);
+          },
+          [&](int m, double pm, double2 cw) {
+            if (it == 0) {
+              k.rh[m] = ri;
+              k.x[m] = 0.0;
+            } else {
+              k.x[m] = fma(omega, k.sh[m], fma(alpha, k.ph[m], k.x[m]));
+              k.r[m] = ri;
+            }
+            pn[m] = pm;
+            kry_restrict(acc, pm, cw);
+            acc[4] = fma(ri, ri, acc[4]);
+          });
+      if (j < n) kry_patches<P>(k, t, sv);
+      kry_block_sums<5, 8>(acc, kry_stage_items<P>(t), [&](int i, double a) {
+        if (i < 4) k.pc[4 * tile + i] = a;
+        else part(kDotRR, tile) = a;
+      });
+    }
+    if (!kry_barrier(st, epoch, status)) return;
+    // the convergence test waits for the next phase's dots (its sum would cost a round trip of
+    // its own), except at the end
+    auto test = [&](double rr, bool last) {
+      sc.rr = rr;
+      if (it == 0) {
+        sc.bb = rr;
+        sc.rho_new = rr;
+        sc.brk = rr == 0.0 || !isfinite(rr);
+      }
+      const bool conv = rr <= sc.tol2 * sc.bb;
+      if (conv || (sc.brk && !last)) {
+        sc.done = conv ? 1 : 2;
+        sc.iters = it;
+      }
+      sc.rho = sc.rho_new;
+    };
+    if (j == n) {
+      kry_sums(k, sc, kDotRR, 0, 0, 0, 1);
+      if (lead) test(sc.dot[0], true);
+      __syncthreads();
+      break;
+    }
+    // ---- B
+    for (int tile = blockIdx.x; tile < k.ntiles; tile += gridDim.x) {
+      const KTile t = one ? t0 : kry_tile(k, tile);
+      KFetch<P> row;
+      kry_fetch<P>(k, t, sv, row);
+      if (!one) kry_load_rows(k, t, a0);
+      kry_coarse(k, a0, vc, zc, cc);
+      kry_gather<P>(k, t, cc, sv, k.ph);
+      double acc[1] = {0.0};
+      kry_apply<P>(k, t, sv, row, [&](int m, double y) {
+        k.v[m] = y;
+        acc[0] = fma(k.rh[m], y, acc[0]);
+      });
+      kry_block_sums<1, 1>(acc, kry_apply_items<P>(t), [&](int, double a) { part(kDotRV, tile) = a; });
+    }
+    if (!kry_barrier(st, epoch, status)) return;
+    // ---- C
+    kry_sums(k, sc, kDotRV, kDotRR, 0, 0, 2);
+    if (lead) {
+      test(sc.dot[1], false);
+      sc.alpha = kry_quot(sc.rho, sc.dot[0]);
+      if (!sc.done && !isfinite(sc.alpha)) {
+        sc.done = 2;
+        sc.iters = it;
+      }
+    }
+    __syncthreads();
+    if (sc.done) break;
+    const double a1 = sc.alpha;
+    for (int tile = blockIdx.x; tile < k.ntiles; tile += gridDim.x) {
+      const KTile t = one ? t0 : kry_tile(k, tile);
+      double acc[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+      kry_stage<P>(
+          k, t, sv, [&](int m) { return fma(-a1, __ldcg(k.v + m), __ldcg(k.r + m)); },
+          [&](int m, double sm, double2 cw) {
+            k.s[m] = sm;
+            kry_restrict(acc, sm, cw);
+            acc[4] = fma(k.rh[m], sm, acc[4]);
+          });
+      kry_patches<P>(k, t, sv);
+      kry_block_sums<5, 8>(acc, kry_stage_items<P>(t), [&](int i, double a) {
+        if (i < 4) k.pc[4 * tile + i] = a;
+        else part(kDotRS, tile) = a;
+      });
+    }
+    if (!kry_barrier(st, epoch, status)) return;
+    // ---- D
+    for (int tile = blockIdx.x; tile < k.ntiles; tile += gridDim.x) {
+      const KTile t = one ? t0 : kry_tile(k, tile);
+      KFetch<P> row;
+      kry_fetch<P>(k, t, sv, row);
+      if (!one) kry_load_rows(k, t, a0);
+      kry_coarse(k, a0, vc, zc, cc);
+      kry_gather<P>(k, t, cc, sv, k.sh);
+      double acc[4] = {0.0, 0.0, 0.0, 0.0};
+      kry_apply<P>(k, t, sv, row, [&](int m, double y) {
+        k.t[m] = y;
+        acc[0] = fma(k.s[m], y, acc[0]);
+        acc[1] = fma(y, y, acc[1]);
+        acc[2] = fma(k.rh[m], y, acc[2]);
+      });
+      kry_block_sums<3, 4>(acc, kry_apply_items<P>(t), [&](int i, double a) { part(i == 0 ? kDotTS : i == 1 ? kDotTT : kDotRT, tile) = a; });
+    }
+    ++it;
+    if (!kry_barrier(st, epoch, status)) return;
+  }
+  if (blockIdx.x == 0 && lead) {
+    st->done = sc.done;
+    st->iters = sc.iters;
+    st->base = it;
+    st->bb = sc.bb;
+    st->rr = sc.rr;
+    st->rho = sc.rho;
+    st->alpha = sc.alpha;
+  }
+}
 
 static inline unsigned nblk(long long n, int bs) { return (unsigned)((n + bs - 1) / bs); }
-
-// n iterations starting at offset 0 from the device's base, then the base's advance
-template <int P>
-static void kry_block(const Kry& k, int n, cudaStream_t s) {
-  constexpr int NL4 = 4 * (P + 1);
-  const unsigned eb = nblk(k.E * NL4, 256), fb = nblk(k.nl, 256);
-  // element patches, coarse restriction and solve, then per multiplier the sum
-  auto precond = [&](const double* x, double* y) {
-    kry_precond_local_kernel<P><<<eb + (unsigned)(k.ncx * k.ncy), 256, 0, s>>>(k, x, eb);
-    kry_coarse_solve_kernel<<<(unsigned)((k.nc + 7) / 8), 256, 0, s>>>(k);
-    kry_precond_gather_kernel<P><<<fb, 256, 0, s>>>(k, y);
-  };
-  for (int j = 0; j < n; ++j) {
-    kry_p_kernel<P><<<kKB, kKT, 0, s>>>(k, j, true);
-    precond(k.p, k.ph);                                                        // p_hat = M^{-1} p
-    kry_matvec_kernel<P><<<kKB, kKT, 0, s>>>(k, k.ph, k.v, k.rh, kDotRV, -1);
-    kry_s_kernel<P><<<kKB, kKT, 0, s>>>(k, j);
-    precond(k.s, k.sh);                                                        // s_hat = M^{-1} s
-    kry_matvec_kernel<P><<<kKB, kKT, 0, s>>>(k, k.sh, k.t, k.s, kDotTS, kDotTT);
-    kry_x_kernel<<<kKB, kKT, 0, s>>>(k, j);
-  }
-  kry_bump_kernel<<<1, 1, 0, s>>>(k.st, n);
-}
-
-// The graph of one block of kCheck iterations for the mesh's current scratch layout,
-// captured once and kept on the handle while the layout stays.
-template <int P>
-static vef_status kry_graph(Mesh& M, const Kry& k, cudaGraphExec_t* out) {
-  if (M.hrt_graph && M.hrt_graph_work == (const void*)M.work && M.hrt_graph_nl == k.nl && M.hrt_graph_p == P) {
-    *out = M.hrt_graph;
-    return VEF_OK;
-  }
-  if (M.hrt_graph) {
-    cudaGraphExecDestroy(M.hrt_graph);
-    M.hrt_graph = nullptr;
-  }
-  cudaStream_t cs;
-  VEF_CUDA_TRY(cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
-  cudaGraph_t g = nullptr;
-  cudaError_t e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
-  if (e == cudaSuccess) {
-    kry_block<P>(k, kCheck, cs);
-    e = cudaStreamEndCapture(cs, &g);
-  }
-  if (e == cudaSuccess) e = cudaGraphInstantiate(&M.hrt_graph, g, 0);
-  if (g) cudaGraphDestroy(g);
-  cudaStreamDestroy(cs);
-  if (e != cudaSuccess) {
-    M.hrt_graph = nullptr;
-    set_last_error(std::string("CUDA error capturing the multiplier iteration: ") + cudaGetErrorString(e));
-    return VEF_ERR_CUDA;
-  }
-  M.hrt_graph_work = M.work;
-  M.hrt_graph_nl = k.nl;
-  M.hrt_graph_p = P;
-  *out = M.hrt_graph;
-  return VEF_OK;
-}
 
 template <int P>
 static vef_status hrt_run(Mesh& M, const HrtIn& in, double tol, int max_iter, double* phi, double* J,
@@ -1419,7 +1720,6 @@ static vef_status hrt_run(Mesh& M, const HrtIn& in, double tol, int max_iter, do
   const size_t per_e = (size_t)S::MM * S::MM + (size_t)S::NJ * S::NL4 + S::NJ + S::N + (size_t)S::NL4 * S::NL4 +
                        S::NL4;
   const size_t vec = (size_t)std::max(1LL, nl);
-  const size_t nsc = (size_t)max_iter + 2;
   const HrtTab tab = make_hrt_tab(P, M.m);
   std::vector<double> refh;
   make_hrt_ref<P>(tab, refh);
@@ -1435,9 +1735,18 @@ static vef_status hrt_run(Mesh& M, const HrtIn& in, double tol, int max_iter, do
     double gw[kMaxP + 1];
     gauss_legendre(P + 1, k.gl, gw);
   }
+  // tiles of the Krylov kernel: a coarse cell each, cut further while a tile's staged vector
+  // with its halo would not fit a CTA's shared memory
+  auto tile_smem = [&] { return (size_t)(k.tw + 2) * (k.th + 2) * 2 * S::NL * sizeof(double); };
+  for (k.sx = k.sy = 1;; ++k.sx, ++k.sy) {
+    k.tw = (k.cx + k.sx - 1) / k.sx;
+    k.th = (k.cy + k.sy - 1) / k.sy;
+    if (tile_smem() <= kTileSmemMax) break;
+  }
+  k.ntiles = k.ncx * k.ncy * k.sx * k.sy;
   const size_t total = per_e * E + 10 * vec + (size_t)(S::NL4 * S::NL4 + S::NL4) * E +
-                       (size_t)nc * nc + (size_t)nc + 20 * (size_t)k.ncx * k.ncy + 2 * vec + (vec + 1) / 2 +
-                       (size_t)kNumDots * kKB + 3 * nsc + sizeof(KState) / sizeof(double) + refh.size() +
+                       (size_t)nc * nc + 16 * (size_t)k.ncx * k.ncy + 4 * (size_t)k.ntiles + 2 * vec +
+                       (size_t)kNumDots * k.ntiles + sizeof(KState) / sizeof(double) + refh.size() +
                        32;   // each of the takes below rounded up to two doubles
   vef_status st = ensure_buffer((void**)&M.work, &M.work_cap, total * sizeof(double));
   if (st != VEF_OK) return st;
@@ -1451,22 +1760,19 @@ static vef_status hrt_run(Mesh& M, const HrtIn& in, double tol, int max_iter, do
   double* He = take((size_t)S::NL4 * S::NL4 * E);
   double* re = take((size_t)S::NL4 * E);
   k.nx = M.nx; k.ny = M.ny; k.nfaces = nfaces; k.nl = nl; k.He = He;
-  k.x = take(vec);   // copied to lambda at the end (the graph keeps one layout)
-  k.r = take(vec); k.rh = take(vec); k.p = take(vec); k.v = take(vec); k.s = take(vec);
+  k.x = lambda && nl > 0 ? lambda : take(vec);
+  k.r = take(vec); k.rh = take(vec); k.p[0] = take(vec); k.p[1] = take(vec); k.v = take(vec); k.s = take(vec);
   k.t = take(vec); k.ph = take(vec); k.sh = take(vec);
   double* Pinv = take((size_t)S::NL4 * S::NL4 * E);
   k.Pinv = Pinv;
   k.z = take((size_t)S::NL4 * E);
   k.E = E;
   k.A0 = take((size_t)nc * nc);
-  k.pc = take((size_t)4 * k.ncx * k.ncy);
-  k.zc = take((size_t)nc);
+  k.pc = take((size_t)4 * k.ntiles);
   double* Acell = take((size_t)16 * k.ncx * k.ncy);
   k.cw = reinterpret_cast<double2*>(take(2 * vec));
-  k.cv = reinterpret_cast<int*>(take((vec + 1) / 2));
-  k.part = take((size_t)kNumDots * kKB);
+  k.part = take((size_t)kNumDots * k.ntiles);
   k.st = reinterpret_cast<KState*>(take(sizeof(KState) / sizeof(double)));
-  k.sc = reinterpret_cast<KScal*>(take(3 * nsc));   // last: its length follows max_iter
   double* refd = take(refh.size());
   // pageable source: the copy has taken the data when the call returns
   VEF_CUDA_TRY(cudaMemcpyAsync(refd, refh.data(), refh.size() * sizeof(double), cudaMemcpyHostToDevice, s));
@@ -1476,7 +1782,7 @@ static vef_status hrt_run(Mesh& M, const HrtIn& in, double tol, int max_iter, do
   VEF_CUDA_TRY(cudaFuncSetAttribute(hrt_local_kernel<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   VEF_CUDA_TRY(cudaFuncSetAttribute(hrt_invert_kernel<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ismem));
   const size_t csmem = (size_t)nc * (nc | 1) * sizeof(float);
-  VEF_CUDA_TRY(cudaFuncSetAttribute(hrt_coarse_invert_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)csmem));
+  VEF_CUDA_TRY(cudaFuncSetAttribute(hrt_coarse_pivot_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)csmem));
   int dev = 0, sms = 0, inv_per_sm = 0;
   VEF_CUDA_TRY(cudaGetDevice(&dev));
   VEF_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
@@ -1497,28 +1803,37 @@ static vef_status hrt_run(Mesh& M, const HrtIn& in, double tol, int max_iter, do
     hrt_coarse_nodes_kernel<P><<<nblk(nl, 256), 256, 0, s>>>(k);
     hrt_coarse_cell_kernel<P><<<(unsigned)(k.ncx * k.ncy), 128, 0, s>>>(k, Acell);
     hrt_coarse_assemble_kernel<<<nblk(nc, 128), 128, 0, s>>>(k, Acell);
-    hrt_coarse_invert_kernel<<<1, kCoarseInvThreads, csmem, s>>>(k);
-    kry_init_kernel<<<kKB, kKT, 0, s>>>(k, tol * tol);
+    int* fallback = (int*)&k.st->done;   // the state is set after the setup
+    hrt_coarse_invert_kernel<<<1, 1024, 0, s>>>(k, fallback);
+    hrt_coarse_pivot_kernel<<<1, kCoarseInvThreads, csmem, s>>>(k, fallback);
     VEF_CUDA_TRY(cudaGetLastError());
-    cudaGraphExec_t graph = nullptr;
-    if (max_iter >= kCheck && (st = kry_graph<P>(M, k, &graph)) != VEF_OK) return st;
-    while (it < max_iter) {
-      const int n = std::min(kCheck, max_iter - it);
-      if (n == kCheck) VEF_CUDA_TRY(cudaGraphLaunch(graph, s));
-      else kry_block<P>(k, n, s);
+    hs.tol2 = tol * tol;
+    VEF_CUDA_TRY(cudaMemcpyAsync(k.st, &hs, sizeof(KState), cudaMemcpyHostToDevice, s));
+    const size_t ksmem = tile_smem();
+    VEF_CUDA_TRY(cudaFuncSetAttribute(kry_solve_kernel<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ksmem));
+    int per_sm = 0;
+    VEF_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kry_solve_kernel<P>, kKT, ksmem));
+    int grid = std::max(1, std::min(k.ntiles, sms * std::max(1, per_sm)));
+    while (!hs.done && it < max_iter) {
+      int n = std::min(kCheck, max_iter - it), check = it + n == max_iter;
+      unsigned int* status = M.dev_status;
+      void* args[] = {&k, &n, &check, &status};
+      // a context limited to part of the device refuses a grid that does not fit it: halve it
+      // (a CTA then takes several tiles)
+      for (;; grid = (grid + 1) / 2) {
+        VEF_CUDA_TRY(cudaMemsetAsync(&k.st->bar, 0, sizeof(unsigned), s));
+        const cudaError_t e = cudaLaunchCooperativeKernel((const void*)kry_solve_kernel<P>, dim3((unsigned)grid),
+                                                          dim3(kKT), args, ksmem, s);
+        if (e == cudaSuccess) break;
+        (void)cudaGetLastError();
+        if (e != cudaErrorCooperativeLaunchTooLarge || grid == 1)
+          return cuda_fail(e, "cudaLaunchCooperativeKernel(kry_solve_kernel)");
+      }
+      VEF_CUDA_TRY(cudaMemcpyAsync(&hs, k.st, sizeof(KState), cudaMemcpyDeviceToHost, s));
+      VEF_CUDA_TRY(cudaStreamSynchronize(s));
       it += n;
-      VEF_CUDA_TRY(cudaGetLastError());
-      VEF_CUDA_TRY(cudaMemcpyAsync(&hs, k.st, sizeof(KState), cudaMemcpyDeviceToHost, s));
-      VEF_CUDA_TRY(cudaStreamSynchronize(s));
-      if (hs.done) break;
-    }
-    if (!hs.done) {   // the test after the last iteration
-      kry_p_kernel<P><<<kKB, kKT, 0, s>>>(k, 0, false);
-      VEF_CUDA_TRY(cudaMemcpyAsync(&hs, k.st, sizeof(KState), cudaMemcpyDeviceToHost, s));
-      VEF_CUDA_TRY(cudaStreamSynchronize(s));
     }
     if (hs.done) it = hs.iters;
-    if (lambda) VEF_CUDA_TRY(cudaMemcpyAsync(lambda, k.x, nl * sizeof(double), cudaMemcpyDeviceToDevice, s));
   }
   {
     KTimer kt(&M, VEF_K_HRT, s);
