@@ -173,6 +173,7 @@ struct Mesh {
   size_t ready_cap = 0;
   void* vef_work = nullptr;      // VEF fixed-point iteration: iterates, moments, closures
   size_t vef_work_cap = 0;
+  void* hrt_ref = nullptr;       // HRT elimination: reference tables (HrtRef in hrt.cu), first use
   ~Mesh();
 };
 

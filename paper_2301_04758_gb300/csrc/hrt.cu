@@ -34,15 +34,15 @@
 // horizontal ((nx-1) ny + j nx + i).
 #include <algorithm>
 #include <cmath>
-#include <vector>
+#include <memory>
 
 #include "device.cuh"
 
 namespace vef {
 namespace {
 
-// 1D tables of one order p and mesh order m: index k < nq is the Gauss point s_k, nq is the
-// point 0 and nq + 1 the point 1.
+// 1D tables of one order p and mesh order m (host): index k < nq is the Gauss point s_k, nq is
+// the point 0 and nq + 1 the point 1.
 struct HrtTab {
   int p, m, nq;
   double w[kMaxNq];                               // Gauss weights
@@ -107,71 +107,28 @@ struct HrtShape {
   static constexpr int NL = P + 1, NL4 = 4 * NL;
 };
 
-// reference RT basis function a at table points (kx, ky): value (2) and d/dxi, d/deta (2 each)
+// the nonzero component of reference RT basis function a (component a / NX) at table points
+// (kx, ky): value, d/dxi, d/deta
 template <int P>
-__host__ __device__ __forceinline__ void rt_ref(const HrtTab& t, int a, int kx, int ky, double v[2], double dxi[2],
-                                       double deta[2]) {
+void rt_ref(const HrtTab& t, int a, int kx, int ky, double& v, double& dxi, double& deta) {
   using S = HrtShape<P>;
-  v[0] = v[1] = dxi[0] = dxi[1] = deta[0] = deta[1] = 0.0;
   if (a < S::NX) {
     const int ax = a % (P + 2), bx = a / (P + 2);
-    v[0] = t.cl[ax][kx] * t.op[bx][ky];
-    dxi[0] = t.dcl[ax][kx] * t.op[bx][ky];
-    deta[0] = t.cl[ax][kx] * t.dop[bx][ky];
+    v = t.cl[ax][kx] * t.op[bx][ky];
+    dxi = t.dcl[ax][kx] * t.op[bx][ky];
+    deta = t.cl[ax][kx] * t.dop[bx][ky];
   } else {
     const int b = a - S::NX, ay = b % (P + 1), by = b / (P + 1);
-    v[1] = t.op[ay][kx] * t.cl[by][ky];
-    dxi[1] = t.dop[ay][kx] * t.cl[by][ky];
-    deta[1] = t.op[ay][kx] * t.dcl[by][ky];
+    v = t.op[ay][kx] * t.cl[by][ky];
+    dxi = t.dop[ay][kx] * t.cl[by][ky];
+    deta = t.op[ay][kx] * t.dcl[by][ky];
   }
-}
-
-// map Jacobian F (row-major [i][k] = d x_i / d xi_k) and second derivatives
-// H[i][k][l] = d^2 x_i / d xi_k d xi_l at table point (kx, ky)
-__device__ __forceinline__ void map_geom(const double* __restrict__ c, const HrtTab& t, int kx, int ky,
-                                         double F[4], double H[8]) {
-  for (int i = 0; i < 4; ++i) F[i] = 0.0;
-  for (int i = 0; i < 8; ++i) H[i] = 0.0;
-  const int q = t.m + 1;
-  for (int b = 0; b < q; ++b)
-    for (int a = 0; a < q; ++a) {
-      const double cx = c[2 * (a + q * b)], cy = c[2 * (a + q * b) + 1];
-      const double dx = t.md[a][kx] * t.mv[b][ky], dy = t.mv[a][kx] * t.md[b][ky];
-      const double xx = t.mdd[a][kx] * t.mv[b][ky], xy = t.md[a][kx] * t.md[b][ky],
-                   yy = t.mv[a][kx] * t.mdd[b][ky];
-      F[0] += cx * dx; F[1] += cx * dy; F[2] += cy * dx; F[3] += cy * dy;
-      H[0] += cx * xx; H[1] += cx * xy; H[2] += cx * xy; H[3] += cx * yy;   // x: [k][l]
-      H[4] += cy * xx; H[5] += cy * xy; H[6] += cy * xy; H[7] += cy * yy;   // y: [k][l]
-    }
 }
 
 // face-point table indices of face f, point k
 __host__ __device__ __forceinline__ void face_pt(int f, int k, int nq, int& kx, int& ky) {
   kx = f == 0 ? k : (f == 1 ? nq + 1 : (f == 2 ? k : nq));
   ky = f == 0 ? nq : (f == 1 ? k : (f == 2 ? nq + 1 : k));
-}
-
-// Eddington tensor (xx, xy, yy) of element e at table point (kx, ky), from the element's
-// nodal phi and P (the DG basis evaluated term by term)
-template <int P>
-__device__ __forceinline__ void eddington_pt(const HrtTab& t, const double* __restrict__ phi,
-                                             const double* __restrict__ Pm, long long En, long long e, int kx,
-                                             int ky, double Eo[3]) {
-  constexpr int Q = P + 1, N = Q * Q;
-  double f = 0, a = 0, b = 0, c = 0;
-#pragma unroll
-  for (int j = 0; j < N; ++j) {
-    const double Bj = t.dg[j % Q][kx] * t.dg[j / Q][ky];
-    const size_t o = (size_t)e * N + j;
-    f += Bj * phi[o];
-    a += Bj * Pm[o];
-    b += Bj * Pm[En + o];
-    c += Bj * Pm[2 * En + o];
-  }
-  const double rf = 1.0 / f;
-  Eo[0] = a * rf;
-  Eo[1] = b * rf;
-  Eo[2] = c * rf;
 }
 
 struct HrtIn {
@@ -197,268 +154,304 @@ struct HrtOut {
   double* re;   // [E][NL4]
 };
 
-// Geometry-independent blocks of the local system, formed once on the host from the same
-// 1D tables: D_ref [n][NJ] = int u div_hat v_hat (the Piola transform makes int u div J dx
-// the reference integral) and C1_ref [4 (p+1)][NJ] = int_f mu (v_hat . n_hat) (the reference
-// normal flux against the multiplier basis; rows of boundary faces are dropped per element).
+// What the elimination needs that depends on no element, formed once per mesh on the host from
+// the 1D tables and kept on the device with the handle.  Points: NQ2 volume points (k1 + NQ k2),
+// then NQ per face.
+template <int P>
 struct HrtRef {
-  const double* D;    // [n][NJ]
-  const double* C1;   // [4 (p+1)][NJ]
+  using S = HrtShape<P>;
+  static constexpr int NPT = S::NQ2 + 4 * S::NQ, NT = S::NJ * (S::NJ + 1) / 2;
+  double D[S::N * S::NJ];           // int u div_hat v_hat (the Piola transform makes int u div J dx this)
+  double C1[S::NL4 * S::NJ];        // int_f mu (v_hat . n_hat) (rows of boundary faces are dropped per element)
+  double rs[S::NQ2][S::NJ];         // the RT functions' nonzero component at the volume points: value,
+  double r0[S::NQ2][S::NJ], r1[S::NQ2][S::NJ];   // d/dxi, d/deta
+  double fv[4 * S::NQ][S::NJ];      // its value at the face points
+  double c2[S::NL4][S::NQ][S::NJ];  // times the multiplier basis: op_t(s_k) fv
+  double bt[NPT][S::N];             // DG basis at the points
+  double w[NPT];                    // w_k1 w_k2, and w_k at the face points
+  double gt[5][(kMaxM + 1) * (kMaxM + 1)][NPT];  // control-point basis: d/dxi, d/deta, second derivatives xx, xy, yy
+  int tri[NT];                      // (r << 8) | c, c >= r: the upper triangle of A
 };
 
 template <int P>
-static void make_hrt_ref(const HrtTab& t, std::vector<double>& out) {
+static void make_hrt_ref(const HrtTab& t, HrtRef<P>& o) {
   using S = HrtShape<P>;
-  constexpr int Q = P + 1, N = S::N, NQ = S::NQ, NJ = S::NJ, NL = S::NL;
-  out.assign((size_t)N * NJ + (size_t)4 * NL * NJ, 0.0);
+  using R = HrtRef<P>;
+  constexpr int Q = P + 1, N = S::N, NQ = S::NQ, NQ2 = S::NQ2, NJ = S::NJ, NL = S::NL;
+  for (int pt = 0; pt < R::NPT; ++pt) {
+    const int f = pt < NQ2 ? -1 : (pt - NQ2) / NQ, k = pt < NQ2 ? 0 : (pt - NQ2) % NQ;
+    int kx = pt % NQ, ky = pt / NQ;
+    if (f >= 0) face_pt(f, k, NQ, kx, ky);
+    o.w[pt] = f < 0 ? t.w[kx] * t.w[ky] : t.w[k];
+    for (int j = 0; j < N; ++j) o.bt[pt][j] = t.dg[j % Q][kx] * t.dg[j / Q][ky];
+    const int q = t.m + 1;
+    for (int c = 0; c < q * q; ++c) {
+      const int a = c % q, b = c / q;
+      o.gt[0][c][pt] = t.md[a][kx] * t.mv[b][ky];
+      o.gt[1][c][pt] = t.mv[a][kx] * t.md[b][ky];
+      o.gt[2][c][pt] = t.mdd[a][kx] * t.mv[b][ky];
+      o.gt[3][c][pt] = t.md[a][kx] * t.md[b][ky];
+      o.gt[4][c][pt] = t.mv[a][kx] * t.mdd[b][ky];
+    }
+    for (int a = 0; a < NJ; ++a) {
+      double v, dx, dy;
+      rt_ref<P>(t, a, kx, ky, v, dx, dy);
+      if (f < 0) {
+        o.rs[pt][a] = v;
+        o.r0[pt][a] = dx;
+        o.r1[pt][a] = dy;
+      } else {
+        o.fv[pt - NQ2][a] = v;
+        for (int tt = 0; tt < NL; ++tt) o.c2[f * NL + tt][k][a] = t.op[tt][k] * v;
+      }
+    }
+  }
   for (int r = 0; r < N; ++r)
     for (int c = 0; c < NJ; ++c) {
       double s = 0.0;
-      for (int k2 = 0; k2 < NQ; ++k2)
-        for (int k1 = 0; k1 < NQ; ++k1) {
-          double vh[2], dx[2], dy[2];
-          rt_ref<P>(t, c, k1, k2, vh, dx, dy);
-          s += t.w[k1] * t.w[k2] * t.dg[r % Q][k1] * t.dg[r / Q][k2] * (dx[0] + dy[1]);
-        }
-      out[(size_t)r * NJ + c] = s;
+      for (int pt = 0; pt < NQ2; ++pt) s += o.w[pt] * o.bt[pt][r] * (c < S::NX ? o.r0[pt][c] : o.r1[pt][c]);
+      o.D[r * NJ + c] = s;
     }
-  double* C1 = out.data() + (size_t)N * NJ;
   for (int f = 0; f < 4; ++f) {
     const double n0 = f == 1 ? 1.0 : (f == 3 ? -1.0 : 0.0), n1 = f == 2 ? 1.0 : (f == 0 ? -1.0 : 0.0);
     for (int tt = 0; tt < NL; ++tt)
       for (int a = 0; a < NJ; ++a) {
         double s = 0.0;
-        for (int k = 0; k < NQ; ++k) {
-          int kx, ky;
-          face_pt(f, k, NQ, kx, ky);
-          double vh[2], dx[2], dy[2];
-          rt_ref<P>(t, a, kx, ky, vh, dx, dy);
-          s += t.w[k] * t.op[tt][k] * (vh[0] * n0 + vh[1] * n1);
-        }
-        C1[(size_t)(f * NL + tt) * NJ + a] = s;
+        for (int k = 0; k < NQ; ++k) s += t.w[k] * o.c2[f * NL + tt][k][a] * (a < S::NX ? n0 : n1);
+        o.C1[(f * NL + tt) * NJ + a] = s;
       }
   }
+  for (int r = 0, i = 0; r < NJ; ++r)
+    for (int c = r; c < NJ; ++c) o.tri[i++] = (r << 8) | c;
 }
 
 template <int P>
 struct HrtSmem {
   using S = HrtShape<P>;
-  static constexpr int NF = 4 * S::NQ;   // face points
+  using R = HrtRef<P>;
+  double rs[S::NQ2][S::NJ];          // HrtRef::rs, read by every product below
   double L[S::MM * S::LD];
-  double vq[S::NQ2][S::NJ][2];       // physical v at the volume points
-  double sg[S::NJ][S::NQ2];          // -w J (grad v : E) at the volume points
-  double wJ[S::NQ2];                 // w J at the volume points
+  double ms[2][S::NQ2][S::NJ];       // sigma_t w J (F^T F / J^2)_{c, comp(a)} times the reference value
+  double sg[S::NQ2][S::NJ];          // -w J (grad v : E) at the volume points
   double C2[S::NJ][S::NL4];
-  double gv[S::NJ], fv[S::N];
+  double gv[S::NJ];
   double ctrl[(kMaxM + 1) * (kMaxM + 1) * 2];
-  // per volume point: F (4, row-major), J, dJ/dxi (2), second derivatives (8), E (3), Q1 (2),
-  // 1 / J
-  double pv[S::NQ2][21];
+  double mom[5][4][S::N];            // nodal phi, P of the element and its face neighbours
+  double geo[R::NPT][10];            // map derivatives: (xi, eta[, xi xi, xi eta, eta eta]) of x and y
+  double ed[S::NQ2 + 8 * S::NQ][4];  // phi and P at the points, then at the face points from outside
+  // per volume point: m00, m01, m11 (sigma_t w J F^T F / J^2), then per component c the weights
+  // of (value, d/dxi, d/deta) in -w J (grad v : E); (w F^T Q1) (2)
+  double pv[S::NQ2][11];
   // per face point: interior faces w (F^T {E} n ds) / J (2); boundary faces (F^T E n^) / J (2),
   // (F^T n^) / J (2), w |n ds| / E_b and 2 w |n ds| J_in / E_b
-  double pf[NF][6];
-  double pa[S::NQ][S::NJ], pb[S::NQ][S::NJ];   // boundary face: v_hat . the two vectors above
+  double pf[4 * S::NQ][6];
 };
 
+// Assembly of one element per CTA at a time.  The work is cut into items that fill warps: the
+// map's derivatives and the moments at the points as small matrix products with the reference
+// tables; then, per point, everything that multiplies a reference basis value, so that A is
+//   A_ab = sum_q [sigma_t w J (F^T F / J^2)_{comp a, comp b} v_a] v_b   (upper triangle),
+// and -w J (grad v_a : E) = K0 v_a + K1 dv_a/dxi + K2 dv_a/deta with three numbers per point
+// and component: an RT function has one nonzero reference component, so its Piola image and
+// gradient need no more.  FP64 issue bounds it: ~35 k lane operations per element at p = 2.
 template <int P>
-__global__ void __launch_bounds__(256, 2)
-hrt_local_kernel(long long E, int nx, int ny, HrtTab tab, HrtRef ref, HrtIn in, HrtOut out, unsigned int* status) {
+__global__ void __launch_bounds__(256, P <= 2 ? 4 : P == 3 ? 3 : 2)
+hrt_local_kernel(long long E, int nx, int ny, int qc, const HrtRef<P>* __restrict__ ref, HrtIn in, HrtOut out) {
   using S = HrtShape<P>;
+  using R = HrtRef<P>;
   constexpr int N = S::N, NQ = S::NQ, NQ2 = S::NQ2, NJ = S::NJ, MM = S::MM, LD = S::LD, NL = S::NL, NL4 = S::NL4;
-  constexpr int NF = HrtSmem<P>::NF;
+  constexpr int NF = 4 * NQ;
   extern __shared__ __align__(16) unsigned char hrt_smem[];
   HrtSmem<P>& sm = *reinterpret_cast<HrtSmem<P>*>(hrt_smem);
   const int tid = threadIdx.x, nth = blockDim.x;
-  // the 1D tables in shared memory: every loop below indexes them per thread, which the
-  // constant bank of a kernel parameter would serve one distinct address at a time
-  __shared__ HrtTab t;
-  static_assert(sizeof(HrtTab) % sizeof(double) == 0, "HrtTab is copied in 8-byte words");
-  for (int i = tid; i < (int)(sizeof(HrtTab) / sizeof(double)); i += nth)
-    reinterpret_cast<double*>(&t)[i] = reinterpret_cast<const double*>(&tab)[i];
-  __syncthreads();
+  for (int i = tid; i < NQ2 * NJ; i += nth) (&sm.rs[0][0])[i] = (&ref->rs[0][0])[i];
   const long long En = E * N;
-  const int qc = (t.m + 1) * (t.m + 1);
   for (long long e = blockIdx.x; e < E; e += gridDim.x) {
     __syncthreads();
+    int nb[4];
+#pragma unroll
+    for (int f = 0; f < 4; ++f) nb[f] = nb_elem(nx, ny, (int)e, f);
+    const bool inner = nb[0] >= 0 && nb[1] >= 0 && nb[2] >= 0 && nb[3] >= 0;
     for (int i = tid; i < 2 * qc; i += nth) sm.ctrl[i] = in.ctrl[(size_t)e * 2 * qc + i];
+    for (int i = tid; i < 20 * N; i += nth) {
+      const int who = i / (4 * N), c = (i / N) & 3, j = i % N;
+      const long long ee = who == 0 ? e : nb[who - 1];
+      if (ee >= 0) sm.mom[who][c][j] = c == 0 ? in.phi[(size_t)ee * N + j] : in.P[(size_t)(c - 1) * En + ee * N + j];
+    }
     const double st = in.sigma_t[e], sa = in.sigma_t[e] - in.sigma_s[e];
     __syncthreads();
-    // (1) once per point: the map's derivatives and the Eddington tensor (both sides of an
-    // interior face, averaged), at the volume and face Gauss points
+    // (1) the map's derivatives (second ones at the volume points only) and the moments at
+    // the points: lanes along the points
+    for (int i = tid; i < NQ2 * 10 + NF * 4; i += nth) {
+      const bool vol = i < NQ2 * 10;
+      const int d = vol ? i / NQ2 : (i - NQ2 * 10) / NF, pt = vol ? i % NQ2 : NQ2 + (i - NQ2 * 10) % NF;
+      const int type = d >> 1, comp = d & 1;
+      double s = 0.0;
+      for (int c = 0; c < qc; ++c) s = fma(ref->gt[type][c][pt], sm.ctrl[2 * c + comp], s);
+      sm.geo[pt][d] = s;
+    }
+    for (int i = tid; i < (NQ2 + 2 * NF) * 4; i += nth) {
+      const int c = i / (NQ2 + 2 * NF), q = i % (NQ2 + 2 * NF);
+      // q: volume points, face points from inside, face points from the neighbour (its own
+      // table points are those of the opposite face)
+      int pt = q, who = 0;
+      if (q >= NQ2 + NF) {
+        const int f = (q - NQ2 - NF) / NQ;
+        who = 1 + f;
+        pt = NQ2 + ((f + 2) & 3) * NQ + (q - NQ2 - NF) % NQ;
+        if (nb[f] < 0) continue;
+      }
+      const double* m = sm.mom[who][c];
+      double s = 0.0;
+#pragma unroll
+      for (int j = 0; j < N; ++j) s = fma(ref->bt[pt][j], m[j], s);
+      sm.ed[q][c] = s;
+    }
+    for (int idx = tid; idx < NL4 * NJ; idx += nth) (&sm.C2[0][0])[idx] = 0.0;
+    __syncthreads();
+    // (2) per point: the numbers that multiply reference basis values
     for (int pt = tid; pt < NQ2 + NF; pt += nth) {
-      const bool vol = pt < NQ2;
-      const int f = vol ? -1 : (pt - NQ2) / NQ, k = vol ? 0 : (pt - NQ2) % NQ;
-      int kx, ky;
-      if (vol) { kx = pt % NQ; ky = pt / NQ; }
-      else face_pt(f, k, NQ, kx, ky);
-      double F[4], H[8];
-      map_geom(sm.ctrl, t, kx, ky, F, H);
-      const double J = F[0] * F[3] - F[1] * F[2];
-      double Eo[3];
-      eddington_pt<P>(t, in.phi, in.P, En, e, kx, ky, Eo);
-      if (vol) {
-        double* g = sm.pv[pt];
-        const double adj[4] = {F[3], -F[1], -F[2], F[0]};
-        for (int i = 0; i < 4; ++i) g[i] = F[i];
-        g[4] = J;
-        for (int l = 0; l < 2; ++l)   // Jacobi's formula: dJ = tr(adj F dF)
-          g[5 + l] = adj[0] * H[0 * 4 + 0 * 2 + l] + adj[1] * H[1 * 4 + 0 * 2 + l] +
-                     adj[2] * H[0 * 4 + 1 * 2 + l] + adj[3] * H[1 * 4 + 1 * 2 + l];
-        for (int i = 0; i < 8; ++i) g[7 + i] = H[i];
-        for (int i = 0; i < 3; ++i) g[15 + i] = Eo[i];
-        double q1x = 0.0, q1y = 0.0;
-        if (in.Q1)
-          for (int j = 0; j < N; ++j) {
-            const double Bj = t.dg[j % (P + 1)][kx] * t.dg[j / (P + 1)][ky];
-            q1x += Bj * in.Q1[(size_t)e * N + j];
-            q1y += Bj * in.Q1[En + (size_t)e * N + j];
+      const double* g = sm.geo[pt];
+      // F = [x_xi x_eta; y_xi y_eta]
+      const double F[4] = {g[0], g[2], g[1], g[3]};
+      const double rJ = 1.0 / (F[0] * F[3] - F[1] * F[2]);
+      const double* o = sm.ed[pt];
+      const double rf = 1.0 / o[0];
+      const double E0 = o[1] * rf, E1 = o[2] * rf, E2 = o[3] * rf;
+      if (pt < NQ2) {
+        double* v = sm.pv[pt];
+        const double w = ref->w[pt], wr = st * w * rJ;   // w J / J^2 = w / J
+        v[0] = wr * (F[0] * F[0] + F[2] * F[2]);
+        v[1] = wr * (F[0] * F[1] + F[2] * F[3]);
+        v[2] = wr * (F[1] * F[1] + F[3] * F[3]);
+        // second derivatives H[i][k][l] = d^2 x_i / dxi_k dxi_l and Jacobi's formula
+        // dJ / dxi_l = tr(adj F dF / dxi_l)
+        const double H[2][2][2] = {{{g[4], g[6]}, {g[6], g[8]}}, {{g[5], g[7]}, {g[7], g[9]}}};
+        // grad v : E = sum_il dv_i / dxi_l B_il / J, B = E adj(F)^T / J; with
+        // dv_i / dxi_l = (H_icl v + F_ic dv_l - dJ_l F_ic v / J) / J and the weight -w J
+        const double adj[2][2] = {{F[3], -F[1]}, {-F[2], F[0]}};
+        double dJ[2], B[2][2];
+#pragma unroll
+        for (int l = 0; l < 2; ++l) {
+          dJ[l] = adj[0][0] * H[0][0][l] + adj[0][1] * H[1][0][l] + adj[1][0] * H[0][1][l] + adj[1][1] * H[1][1][l];
+          B[0][l] = -w * rJ * (adj[l][0] * E0 + adj[l][1] * E1);
+          B[1][l] = -w * rJ * (adj[l][0] * E1 + adj[l][1] * E2);
+        }
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+          const double f0 = F[c], f1 = F[2 + c];
+          double k0 = 0.0;
+#pragma unroll
+          for (int l = 0; l < 2; ++l) {
+            const double t = dJ[l] * rJ;
+            k0 += B[0][l] * (H[0][c][l] - t * f0) + B[1][l] * (H[1][c][l] - t * f1);
+            v[4 + 3 * c + l] = B[0][l] * f0 + B[1][l] * f1;
           }
-        g[18] = q1x;
-        g[19] = q1y;
-        g[20] = 1.0 / J;
+          v[3 + 3 * c] = k0;
+        }
+        if (in.Q1) {   // int v . Q1: w J (F v / J) . Q1
+          double q1x = 0.0, q1y = 0.0;
+          for (int j = 0; j < N; ++j) {
+            q1x += ref->bt[pt][j] * in.Q1[(size_t)e * N + j];
+            q1y += ref->bt[pt][j] * in.Q1[En + (size_t)e * N + j];
+          }
+          v[9] = w * (F[0] * q1x + F[2] * q1y);
+          v[10] = w * (F[1] * q1x + F[3] * q1y);
+        }
       } else {
-        double* o = sm.pf[pt - NQ2];
+        const int fp = pt - NQ2, f = fp / NQ, k = fp % NQ;
+        double* r = sm.pf[fp];
         const double* nd = in.nds + (((size_t)e * 4 + f) * NQ + k) * 2;
-        const int nb = nb_elem(nx, ny, (int)e, f);
-        if (nb >= 0) {
-          int nkx, nky;
-          face_pt((f + 2) & 3, k, NQ, nkx, nky);
-          double Enb[3];
-          eddington_pt<P>(t, in.phi, in.P, En, nb, nkx, nky, Enb);
-          const double a00 = 0.5 * (Eo[0] + Enb[0]), a01 = 0.5 * (Eo[1] + Enb[1]), a11 = 0.5 * (Eo[2] + Enb[2]);
+        const double w = ref->w[pt];
+        if (nb[f] >= 0) {
+          const double* on = sm.ed[pt + NF];
+          const double rn = 1.0 / on[0];
+          const double a00 = 0.5 * (E0 + on[1] * rn), a01 = 0.5 * (E1 + on[2] * rn), a11 = 0.5 * (E2 + on[3] * rn);
           const double En0 = a00 * nd[0] + a01 * nd[1], En1 = a01 * nd[0] + a11 * nd[1];
           // v_a . {E} n ds = v_hat_a . F^T ({E} n ds) / J
-          o[0] = t.w[k] * (F[0] * En0 + F[2] * En1) / J;
-          o[1] = t.w[k] * (F[1] * En0 + F[3] * En1) / J;
+          r[0] = w * (F[0] * En0 + F[2] * En1) * rJ;
+          r[1] = w * (F[1] * En0 + F[3] * En1) * rJ;
         } else {
           const long long bf = bface(nx, ny, (int)e, f);
           const double ln = sqrt(nd[0] * nd[0] + nd[1] * nd[1]);
           const double un0 = nd[0] / ln, un1 = nd[1] / ln;
-          const double En0 = Eo[0] * un0 + Eo[1] * un1, En1 = Eo[1] * un0 + Eo[2] * un1;
+          const double En0 = E0 * un0 + E1 * un1, En1 = E1 * un0 + E2 * un1;
           const double eb = in.Eb[bf * NQ + k];
-          o[0] = (F[0] * En0 + F[2] * En1) / J;
-          o[1] = (F[1] * En0 + F[3] * En1) / J;
-          o[2] = (F[0] * un0 + F[2] * un1) / J;
-          o[3] = (F[1] * un0 + F[3] * un1) / J;
-          o[4] = t.w[k] * ln / eb;
-          o[5] = 2.0 * t.w[k] * ln * in.Jin[bf * NQ + k] / eb;
+          r[0] = (F[0] * En0 + F[2] * En1) * rJ;
+          r[1] = (F[1] * En0 + F[3] * En1) * rJ;
+          r[2] = (F[0] * un0 + F[2] * un1) * rJ;
+          r[3] = (F[1] * un0 + F[3] * un1) * rJ;
+          r[4] = w * ln / eb;
+          r[5] = 2.0 * w * ln * in.Jin[bf * NQ + k] / eb;
         }
       }
     }
     __syncthreads();
-    // (2) per (volume point, basis function): the physical v and -w J (grad v : E)
+    // (3) per (volume point, basis function); the multiplier couplings of the interior faces
     for (int idx = tid; idx < NQ2 * NJ; idx += nth) {
-      const int q = idx / NJ, a = idx % NJ, k1 = q % NQ, k2 = q / NQ;
-      const double* g = sm.pv[q];
-      const double F[4] = {g[0], g[1], g[2], g[3]};
-      const double J = g[4], rJ = g[20];
-      const double adj[4] = {F[3], -F[1], -F[2], F[0]};
-      double vh[2], dx[2], dy[2];
-      rt_ref<P>(t, a, k1, k2, vh, dx, dy);
-      double v[2], dv[2][2];   // dv[i][l] = d v_i / d xi_l
-      for (int i = 0; i < 2; ++i) v[i] = (F[2 * i] * vh[0] + F[2 * i + 1] * vh[1]) * rJ;
-      for (int l = 0; l < 2; ++l) {
-        const double* dvh = l == 0 ? dx : dy;
-        for (int i = 0; i < 2; ++i) {
-          const double dFv = g[7 + i * 4 + 0 * 2 + l] * vh[0] + g[7 + i * 4 + 1 * 2 + l] * vh[1];
-          const double Fdv = F[2 * i] * dvh[0] + F[2 * i + 1] * dvh[1];
-          dv[i][l] = (dFv + Fdv - g[5 + l] * v[i]) * rJ;
-        }
-      }
-      // grad v = dv F^{-1}, F^{-1} = adj / J; grad v : E
-      double gE = 0.0;
-      for (int i = 0; i < 2; ++i)
-        for (int mcol = 0; mcol < 2; ++mcol) {
-          const double gim = (dv[i][0] * adj[0 * 2 + mcol] + dv[i][1] * adj[1 * 2 + mcol]) * rJ;
-          const double Eim = (i == mcol) ? (i == 0 ? g[15] : g[17]) : g[16];
-          gE += gim * Eim;
-        }
-      const double w = t.w[k1] * t.w[k2];
-      sm.vq[q][a][0] = v[0];
-      sm.vq[q][a][1] = v[1];
-      sm.sg[a][q] = -w * J * gE;
-      if (a == 0) sm.wJ[q] = w * J;
+      const int q = idx / NJ, a = idx % NJ, c = a < S::NX ? 0 : 1;
+      const double* v = sm.pv[q];
+      const double s = sm.rs[q][a];
+      sm.ms[0][q][a] = v[c] * s;
+      sm.ms[1][q][a] = v[1 + c] * s;
+      sm.sg[q][a] = fma(v[3 + 3 * c], s, fma(v[4 + 3 * c], ref->r0[q][a], v[5 + 3 * c] * ref->r1[q][a]));
     }
-    for (int idx = tid; idx < NL4 * NJ; idx += nth) (&sm.C2[0][0])[idx] = 0.0;
-    __syncthreads();
-    // (3) A (symmetric: one triangle computed), G, D (reference), sigma_a M, f, g
-    for (int idx = tid; idx < MM * MM; idx += nth) {
-      const int r = idx / MM, c = idx % MM;
-      if (r < NJ && c < NJ) {
-        if (c < r) continue;
-        double val = 0.0;
-        for (int q = 0; q < NQ2; ++q)
-          val += sm.wJ[q] * (sm.vq[q][r][0] * sm.vq[q][c][0] + sm.vq[q][r][1] * sm.vq[q][c][1]);
-        val *= st;
-        sm.L[r * LD + c] = val;
-        sm.L[c * LD + r] = val;
-        continue;
-      }
-      double val;
-      if (r < NJ) {
-        const int cc = c - NJ;
-        val = 0.0;
-        for (int q = 0; q < NQ2; ++q)
-          val += sm.sg[r][q] * t.dg[cc % (P + 1)][q % NQ] * t.dg[cc / (P + 1)][q / NQ];
-      } else if (c < NJ) {
-        val = ref.D[(r - NJ) * NJ + c];
-      } else {
-        val = sa * in.Mm[((size_t)e * N + (r - NJ)) * N + (c - NJ)];
-      }
-      sm.L[r * LD + c] = val;
-    }
-    for (int c = tid; c < N; c += nth) {
+    for (int idx = tid; idx < NL4 * NJ; idx += nth) {
+      const int ft = idx / NJ, a = idx % NJ, f = ft / NL, c = a < S::NX ? 0 : 1;
+      if (nb[f] < 0) continue;
       double s = 0.0;
-      for (int j = 0; j < N; ++j) s += in.Mm[((size_t)e * N + c) * N + j] * in.Q0[(size_t)e * N + j];
-      sm.fv[c] = s;
-    }
-    for (int a = tid; a < NJ; a += nth) {
-      double s = 0.0;
-      if (in.Q1)
-        for (int q = 0; q < NQ2; ++q)
-          s += sm.wJ[q] * (sm.vq[q][a][0] * sm.pv[q][18] + sm.vq[q][a][1] * sm.pv[q][19]);
-      sm.gv[a] = s;
+#pragma unroll
+      for (int k = 0; k < NQ; ++k) s = fma(ref->c2[ft][k][a], sm.pf[f * NQ + k][c], s);
+      sm.C2[a][ft] = s;
     }
     __syncthreads();
-    // (4) faces: multiplier couplings on interior faces, Miften-Larsen terms on boundary faces
-    for (int f = 0; f < 4; ++f) {
-      const double* o0 = sm.pf[f * NQ];
-      if (nb_elem(nx, ny, (int)e, f) >= 0) {
-        for (int idx = tid; idx < NJ * NL; idx += nth) {
-          const int a = idx / NL, tt = idx % NL;
-          double c2 = 0.0;
-          for (int k = 0; k < NQ; ++k) {
-            int kx, ky;
-            face_pt(f, k, NQ, kx, ky);
-            double vh[2], dx[2], dy[2];
-            rt_ref<P>(t, a, kx, ky, vh, dx, dy);
-            c2 += t.op[tt][k] * (vh[0] * o0[6 * k] + vh[1] * o0[6 * k + 1]);
-          }
-          sm.C2[a][f * NL + tt] = c2;
-        }
+    // (4) A (upper triangle, mirrored), G, D (reference), sigma_a M, f, g
+    for (int idx = tid; idx < R::NT; idx += nth) {
+      const int rc = ref->tri[idx], r = rc >> 8, c = rc & 0xff, cc = c < S::NX ? 0 : 1;
+      double s = 0.0;
+#pragma unroll 4
+      for (int q = 0; q < NQ2; ++q) s = fma(sm.ms[cc][q][r], sm.rs[q][c], s);
+      sm.L[r * LD + c] = s;
+      sm.L[c * LD + r] = s;
+    }
+    for (int idx = tid; idx < NJ * N; idx += nth) {
+      const int c = idx / NJ, a = idx % NJ;
+      double s = 0.0;
+#pragma unroll 4
+      for (int q = 0; q < NQ2; ++q) s = fma(sm.sg[q][a], ref->bt[q][c], s);
+      sm.L[a * LD + NJ + c] = s;
+      sm.L[(NJ + c) * LD + a] = ref->D[idx];
+    }
+    for (int idx = tid; idx < N * N; idx += nth)
+      sm.L[(NJ + idx / N) * LD + NJ + idx % N] = sa * in.Mm[(size_t)e * N * N + idx];
+    for (int c = tid; c < N + NJ; c += nth) {
+      double s = 0.0;
+      if (c < N) {
+        for (int j = 0; j < N; ++j) s += in.Mm[((size_t)e * N + c) * N + j] * in.Q0[(size_t)e * N + j];
+        out.f[(size_t)e * N + c] = s;
       } else {
-        for (int idx = tid; idx < NQ * NJ; idx += nth) {
-          const int k = idx / NJ, a = idx % NJ;
-          int kx, ky;
-          face_pt(f, k, NQ, kx, ky);
-          double vh[2], dx[2], dy[2];
-          rt_ref<P>(t, a, kx, ky, vh, dx, dy);
-          const double* o = o0 + 6 * k;
-          sm.pa[k][a] = vh[0] * o[0] + vh[1] * o[1];
-          sm.pb[k][a] = vh[0] * o[2] + vh[1] * o[3];
-        }
-        __syncthreads();
-        for (int idx = tid; idx < NJ * NJ + NJ; idx += nth) {
-          const int a = idx < NJ * NJ ? idx / NJ : idx - NJ * NJ;
-          const int b = idx < NJ * NJ ? idx % NJ : -1;
-          double s = 0.0;
-          if (b >= 0) {
-            for (int k = 0; k < NQ; ++k) s += o0[6 * k + 4] * sm.pa[k][a] * sm.pb[k][b];
-            sm.L[a * LD + b] += s;
-          } else {
-            for (int k = 0; k < NQ; ++k) s += o0[6 * k + 5] * sm.pa[k][a];
-            sm.gv[a] += s;
-          }
+        const int a = c - N, k = a < S::NX ? 9 : 10;
+        if (in.Q1)
+          for (int q = 0; q < NQ2; ++q) s += sm.rs[q][a] * sm.pv[q][k];
+        sm.gv[a] = s;
+      }
+    }
+    __syncthreads();
+    // (5) Miften-Larsen terms of the boundary faces
+    for (int f = 0; f < 4 && !inner; ++f) {
+      if (nb[f] >= 0) continue;
+      const double (*o)[6] = sm.pf + f * NQ;
+      for (int idx = tid; idx < NJ * NJ + NJ; idx += nth) {
+        const int a = idx < NJ * NJ ? idx / NJ : idx - NJ * NJ, b = idx < NJ * NJ ? idx % NJ : -1;
+        const int ca = a < S::NX ? 0 : 1, cb = b < S::NX ? 0 : 1;
+        double s = 0.0;
+        if (b >= 0) {
+          for (int k = 0; k < NQ; ++k)
+            s += o[k][4] * (ref->fv[f * NQ + k][a] * o[k][ca]) * (ref->fv[f * NQ + k][b] * o[k][2 + cb]);
+          sm.L[a * LD + b] += s;
+        } else {
+          for (int k = 0; k < NQ; ++k) s += o[k][5] * (ref->fv[f * NQ + k][a] * o[k][ca]);
+          sm.gv[a] += s;
         }
       }
       __syncthreads();
@@ -468,134 +461,192 @@ hrt_local_kernel(long long E, int nx, int ny, HrtTab tab, HrtRef ref, HrtIn in, 
       out.Li[(size_t)e * MM * MM + idx] = sm.L[(idx / MM) * LD + idx % MM];
     for (int idx = tid; idx < NJ * NL4; idx += nth) out.C2[(size_t)e * NJ * NL4 + idx] = (&sm.C2[0][0])[idx];
     for (int a = tid; a < NJ; a += nth) out.g[(size_t)e * NJ + a] = sm.gv[a];
-    for (int c = tid; c < N; c += nth) out.f[(size_t)e * N + c] = sm.fv[c];
   }
 }
 
 // Inversion of the assembled local systems and the element's share of the reduced system,
-// apart from the assembly so that it runs many CTAs per SM: its Gauss-Jordan steps are
-// short and separated by barriers, and only the number of CTAs in flight hides them.
+// apart from the assembly so that it runs many CTAs per SM.  Gauss-Jordan with the matrix in
+// registers (entry idx = i MM + j on thread idx mod T): per step the pivot's row and column
+// are published in shared memory and every entry takes one FMA, a = R_j (-c_i) + a with
+// R = row / pivot, where the pivot's own row and column start from zero (R_k = 1 / pivot,
+// -c_k = 1), so no lane of a warp takes another path.  The diagonal pivots are taken in
+// order: A is positive definite for sigma_t > 0, and so is the Schur complement
+// sigma_a M - D A^{-1} G, with G close to -E : D^T.  A system with a pivot below
+// 2^-kHrtPivotFloor of its row's largest entry, or not finite, is inverted again with partial
+// pivoting (the slow path, from the assembled system).
+constexpr int kHrtPivotFloor = 26;
 template <int P>
 struct HrtInvSmem {
   using S = HrtShape<P>;
   double L[S::MM * S::LD];
-  double C1[S::NL4][S::NJ];
   double C2[S::NJ][S::NL4];
-  double gv[S::NJ], fv[S::N];
-  double T1[S::NJ][S::NL4];          // W C2
-  double u[S::NJ];                   // W g + X f
+  double gf[S::MM];                  // g, f
+  double T1[S::NL4][S::NL4];         // rows of W C2 at the face unknowns
+  double u[S::NL4];                  // W g + X f there
+  double row[S::MM], col[S::MM];     // the pivot's row and column, as published
+  double R[S::MM], nc[S::MM];        // row / pivot and -column
   double colk[S::MM];
-  double inv;                        // reciprocal of the current pivot
+  double inv;                        // reciprocal of the current pivot (slow path)
+  int scale[S::MM];                  // high word of each row's largest magnitude
   int perm[S::MM];
   int piv;
 };
+template <int P> struct HrtInvShape {
+  static constexpr int T = P <= 2 ? 128 : 256, NR = (HrtShape<P>::MM * HrtShape<P>::MM + T - 1) / T;
+};
 
 template <int P>
-__global__ void __launch_bounds__(128)
-hrt_invert_kernel(long long E, int nx, int ny, HrtRef ref, HrtOut out, unsigned int* status) {
+__global__ void __launch_bounds__(HrtInvShape<P>::T)
+hrt_invert_kernel(long long E, int nx, int ny, const HrtRef<P>* __restrict__ ref, HrtOut out, unsigned int* status) {
   using S = HrtShape<P>;
-  constexpr int N = S::N, NJ = S::NJ, MM = S::MM, LD = S::LD, NL = S::NL, NL4 = S::NL4;
+  constexpr int N = S::N, NJ = S::NJ, MM = S::MM, LD = S::LD, NL = S::NL, NL4 = S::NL4, NX = S::NX;
+  constexpr int T = HrtInvShape<P>::T, NR = HrtInvShape<P>::NR;
   extern __shared__ __align__(16) unsigned char hrt_inv_smem[];
   HrtInvSmem<P>& sm = *reinterpret_cast<HrtInvSmem<P>*>(hrt_inv_smem);
-  const int tid = threadIdx.x, nth = blockDim.x;
+  const int tid = threadIdx.x, nth = T;
+  // the RT unknown with a normal flux on face f at tangential node b (C1's columns)
+  auto face_unknown = [](int f, int b) {
+    return f == 3 ? (P + 2) * b : f == 1 ? P + 1 + (P + 2) * b : f == 0 ? NX + b : NX + b + (P + 1) * (P + 1);
+  };
   for (long long e = blockIdx.x; e < E; e += gridDim.x) {
     __syncthreads();
-    for (int idx = tid; idx < MM * MM; idx += nth)
-      sm.L[(idx / MM) * LD + idx % MM] = out.Li[(size_t)e * MM * MM + idx];
-    for (int idx = tid; idx < NL4 * NJ; idx += nth) {
-      const int r = idx / NJ;
-      (&sm.C1[0][0])[idx] = nb_elem(nx, ny, (int)e, r / NL) >= 0 ? ref.C1[idx] : 0.0;
-      (&sm.C2[0][0])[idx] = out.C2[(size_t)e * NJ * NL4 + idx];
-    }
-    for (int a = tid; a < NJ; a += nth) sm.gv[a] = out.g[(size_t)e * NJ + a];
-    for (int c = tid; c < N; c += nth) sm.fv[c] = out.f[(size_t)e * N + c];
+    for (int i = tid; i < MM; i += nth) sm.scale[i] = 0;
+    for (int idx = tid; idx < NL4 * NJ; idx += nth) (&sm.C2[0][0])[idx] = out.C2[(size_t)e * NJ * NL4 + idx];
+    for (int a = tid; a < MM; a += nth) sm.gf[a] = a < NJ ? out.g[(size_t)e * NJ + a] : out.f[(size_t)e * N + a - NJ];
+    double* Lg = out.Li + (size_t)e * MM * MM;
+    double a[NR];
     __syncthreads();
-    // in-place Gauss-Jordan inversion of L with partial pivoting
+#pragma unroll
+    for (int r = 0; r < NR; ++r) {
+      const int idx = tid + r * T, i = idx / MM;
+      a[r] = idx < MM * MM ? Lg[idx] : 0.0;
+      if (idx < MM * MM) atomicMax(&sm.scale[i], __double2hiint(a[r]) & 0x7fffffff);
+    }
+    bool bad = false;
     for (int k = 0; k < MM; ++k) {
-      if (tid < 32) {
-        double best = -1.0;
-        int bi = k;
-        for (int i = k + tid; i < MM; i += 32) {
-          const double v = fabs(sm.L[i * LD + k]);
-          if (v > best) { best = v; bi = i; }
-        }
-        for (int off = 16; off > 0; off >>= 1) {
-          const double ob = __shfl_xor_sync(0xffffffffu, best, off);
-          const int oi = __shfl_xor_sync(0xffffffffu, bi, off);
-          if (ob > best || (ob == best && oi < bi)) { best = ob; bi = oi; }
-        }
-        if (tid == 0) {
-          sm.piv = bi;
-          sm.perm[k] = bi;
-          sm.inv = 1.0 / sm.L[bi * LD + k];   // one FP64 division per step, not one per thread
-          if (!(best > 1e-300)) atomicOr(status, kDevSingular);
+#pragma unroll
+      for (int r = 0; r < NR; ++r) {
+        const int idx = tid + r * T, i = idx / MM, j = idx - i * MM;
+        if (i == k) sm.row[j] = a[r];
+        if (j == k && i < MM) sm.col[i] = a[r];
+      }
+      __syncthreads();
+      if (tid < (MM + 31) / 32 * 32) {
+        const double piv = sm.row[k];
+        const int mag = __double2hiint(piv) & 0x7fffffff;
+        bad = bad || mag < sm.scale[k] - (kHrtPivotFloor << 20) || mag >= (2000 << 20) || mag < (50 << 20);
+        const double inv = pivot_rcp(piv);
+        if (tid < MM) {
+          sm.R[tid] = tid == k ? inv : sm.row[tid] * inv;
+          sm.nc[tid] = tid == k ? 1.0 : -sm.col[tid];
         }
       }
       __syncthreads();
-      const int pr = sm.piv;
-      if (pr != k)
-        for (int j = tid; j < MM; j += nth) {
-          const double tmp = sm.L[k * LD + j];
-          sm.L[k * LD + j] = sm.L[pr * LD + j];
-          sm.L[pr * LD + j] = tmp;
-        }
-      __syncthreads();
-      const double inv = sm.inv;
-      for (int i = tid; i < MM; i += nth) sm.colk[i] = sm.L[i * LD + k];
-      __syncthreads();
-      for (int j = tid; j < MM; j += nth)
-        if (j != k) sm.L[k * LD + j] *= inv;
-      __syncthreads();
-      for (int idx = tid; idx < MM * MM; idx += nth) {
-        const int i = idx / MM, j = idx % MM;
-        if (i == k) continue;
-        if (j == k) sm.L[i * LD + k] = -sm.colk[i] * inv;
-        else sm.L[i * LD + j] -= sm.colk[i] * sm.L[k * LD + j];
+#pragma unroll
+      for (int r = 0; r < NR; ++r) {
+        const int idx = tid + r * T, i = idx / MM, j = idx - i * MM;
+        const double old = i == k || j == k ? 0.0 : a[r];
+        if (idx < MM * MM) a[r] = fma(sm.nc[i], sm.R[j], old);
       }
-      if (tid == 0) sm.L[k * LD + k] = inv;
-      __syncthreads();
     }
-    for (int k = MM - 1; k >= 0; --k) {   // undo the row interchanges as column interchanges
-      const int pr = sm.perm[k];
-      if (pr != k)
-        for (int i = tid; i < MM; i += nth) {
-          const double tmp = sm.L[i * LD + k];
-          sm.L[i * LD + k] = sm.L[i * LD + pr];
-          sm.L[i * LD + pr] = tmp;
+    if (!__syncthreads_or(bad)) {
+#pragma unroll
+      for (int r = 0; r < NR; ++r) {
+        const int idx = tid + r * T;
+        if (idx < MM * MM) {
+          sm.L[(idx / MM) * LD + idx % MM] = a[r];
+          Lg[idx] = a[r];
         }
+      }
       __syncthreads();
+    } else {
+      for (int idx = tid; idx < MM * MM; idx += nth) sm.L[(idx / MM) * LD + idx % MM] = Lg[idx];
+      __syncthreads();
+      for (int k = 0; k < MM; ++k) {
+        if (tid < 32) {
+          double best = -1.0;
+          int bi = k;
+          for (int i = k + tid; i < MM; i += 32) {
+            const double v = fabs(sm.L[i * LD + k]);
+            if (v > best) { best = v; bi = i; }
+          }
+          for (int off = 16; off > 0; off >>= 1) {
+            const double ob = __shfl_xor_sync(0xffffffffu, best, off);
+            const int oi = __shfl_xor_sync(0xffffffffu, bi, off);
+            if (ob > best || (ob == best && oi < bi)) { best = ob; bi = oi; }
+          }
+          if (tid == 0) {
+            sm.piv = bi;
+            sm.perm[k] = bi;
+            sm.inv = 1.0 / sm.L[bi * LD + k];   // one FP64 division per step, not one per thread
+            if (!(best > 1e-300)) atomicOr(status, kDevSingular);
+          }
+        }
+        __syncthreads();
+        const int pr = sm.piv;
+        if (pr != k)
+          for (int j = tid; j < MM; j += nth) {
+            const double tmp = sm.L[k * LD + j];
+            sm.L[k * LD + j] = sm.L[pr * LD + j];
+            sm.L[pr * LD + j] = tmp;
+          }
+        __syncthreads();
+        const double inv = sm.inv;
+        for (int i = tid; i < MM; i += nth) sm.colk[i] = sm.L[i * LD + k];
+        __syncthreads();
+        for (int j = tid; j < MM; j += nth)
+          if (j != k) sm.L[k * LD + j] *= inv;
+        __syncthreads();
+        for (int idx = tid; idx < MM * MM; idx += nth) {
+          const int i = idx / MM, j = idx % MM;
+          if (i == k) continue;
+          if (j == k) sm.L[i * LD + k] = -sm.colk[i] * inv;
+          else sm.L[i * LD + j] -= sm.colk[i] * sm.L[k * LD + j];
+        }
+        if (tid == 0) sm.L[k * LD + k] = inv;
+        __syncthreads();
+      }
+      for (int k = MM - 1; k >= 0; --k) {   // undo the row interchanges as column interchanges
+        const int pr = sm.perm[k];
+        if (pr != k)
+          for (int i = tid; i < MM; i += nth) {
+            const double tmp = sm.L[i * LD + k];
+            sm.L[i * LD + k] = sm.L[i * LD + pr];
+            sm.L[i * LD + pr] = tmp;
+          }
+        __syncthreads();
+      }
+      for (int idx = tid; idx < MM * MM; idx += nth) Lg[idx] = sm.L[(idx / MM) * LD + idx % MM];
     }
-    // W C2 and W g + X f, then H_e = C1 (W C2) and r_e = C1 (W g + X f)
-    for (int idx = tid; idx < NJ * NL4 + NJ; idx += nth) {
-      if (idx < NJ * NL4) {
-        const int a = idx / NL4, c = idx % NL4;
-        double s = 0.0;
-        for (int b = 0; b < NJ; ++b) s += sm.L[a * LD + b] * sm.C2[b][c];
-        sm.T1[a][c] = s;
+    // W C2 and W g + X f at the unknowns with a normal flux on a face (the others have zero
+    // columns in C1), then H_e = C1 (W C2) and r_e = C1 (W g + X f)
+    for (int idx = tid; idx < NL4 * NL4 + NL4; idx += nth) {
+      const int r = idx < NL4 * NL4 ? idx / NL4 : idx - NL4 * NL4;
+      const double* Lr = sm.L + face_unknown(r / NL, r % NL) * LD;
+      double s = 0.0;
+      if (idx < NL4 * NL4) {
+        const int c = idx % NL4;
+        for (int b = 0; b < NJ; ++b) s = fma(Lr[b], sm.C2[b][c], s);
+        sm.T1[r][c] = s;
       } else {
-        const int a = idx - NJ * NL4;
-        double s = 0.0;
-        for (int b = 0; b < NJ; ++b) s += sm.L[a * LD + b] * sm.gv[b];
-        for (int c = 0; c < N; ++c) s += sm.L[a * LD + NJ + c] * sm.fv[c];
-        sm.u[a] = s;
+        for (int b = 0; b < MM; ++b) s = fma(Lr[b], sm.gf[b], s);
+        sm.u[r] = s;
       }
     }
     __syncthreads();
     for (int idx = tid; idx < NL4 * NL4 + NL4; idx += nth) {
-      if (idx < NL4 * NL4) {
-        const int r = idx / NL4, c = idx % NL4;
-        double s = 0.0;
-        for (int a = 0; a < NJ; ++a) s += sm.C1[r][a] * sm.T1[a][c];
-        out.He[(size_t)e * NL4 * NL4 + idx] = s;
-      } else {
-        const int r = idx - NL4 * NL4;
-        double s = 0.0;
-        for (int a = 0; a < NJ; ++a) s += sm.C1[r][a] * sm.u[a];
-        out.re[(size_t)e * NL4 + r] = s;
+      const int r = idx < NL4 * NL4 ? idx / NL4 : idx - NL4 * NL4, f = r / NL;
+      double s = 0.0;
+      if (nb_elem(nx, ny, (int)e, f) >= 0) {
+#pragma unroll
+        for (int b = 0; b < NL; ++b) {
+          const double c1 = ref->C1[r * NJ + face_unknown(f, b)];
+          s = fma(c1, idx < NL4 * NL4 ? sm.T1[f * NL + b][idx % NL4] : sm.u[f * NL + b], s);
+        }
       }
+      if (idx < NL4 * NL4) out.He[(size_t)e * NL4 * NL4 + idx] = s;
+      else out.re[(size_t)e * NL4 + r] = s;
     }
-    for (int idx = tid; idx < MM * MM; idx += nth)
-      out.Li[(size_t)e * MM * MM + idx] = sm.L[(idx / MM) * LD + idx % MM];
   }
 }
 
@@ -1720,9 +1771,22 @@ static vef_status hrt_run(Mesh& M, const HrtIn& in, double tol, int max_iter, do
   const size_t per_e = (size_t)S::MM * S::MM + (size_t)S::NJ * S::NL4 + S::NJ + S::N + (size_t)S::NL4 * S::NL4 +
                        S::NL4;
   const size_t vec = (size_t)std::max(1LL, nl);
-  const HrtTab tab = make_hrt_tab(P, M.m);
-  std::vector<double> refh;
-  make_hrt_ref<P>(tab, refh);
+  if (!M.hrt_ref) {   // the reference tables, once per mesh
+    auto refh = std::make_unique<HrtRef<P>>();
+    make_hrt_ref<P>(make_hrt_tab(P, M.m), *refh);
+    void* dev = nullptr;
+    size_t cap = 0;
+    vef_status st = ensure_buffer(&dev, &cap, sizeof(HrtRef<P>));
+    if (st != VEF_OK) return st;
+    cudaError_t ce = cudaMemcpyAsync(dev, refh.get(), sizeof(HrtRef<P>), cudaMemcpyHostToDevice, s);
+    if (ce == cudaSuccess) ce = cudaStreamSynchronize(s);
+    if (ce != cudaSuccess) {
+      cudaFree(dev);
+      return cuda_fail(ce, "copying the HRT reference tables");
+    }
+    M.hrt_ref = dev;
+  }
+  const HrtRef<P>* ref = (const HrtRef<P>*)M.hrt_ref;
   // the coarse grid: at most kCoarseMaxCells cells per direction
   Kry k{};
   k.cx = (M.nx + kCoarseMaxCells - 1) / kCoarseMaxCells;
@@ -1746,7 +1810,7 @@ static vef_status hrt_run(Mesh& M, const HrtIn& in, double tol, int max_iter, do
   k.ntiles = k.ncx * k.ncy * k.sx * k.sy;
   const size_t total = per_e * E + 10 * vec + (size_t)(S::NL4 * S::NL4 + S::NL4) * E +
                        (size_t)nc * nc + 16 * (size_t)k.ncx * k.ncy + 4 * (size_t)k.ntiles + 2 * vec +
-                       (size_t)kNumDots * k.ntiles + sizeof(KState) / sizeof(double) + refh.size() +
+                       (size_t)kNumDots * k.ntiles + sizeof(KState) / sizeof(double) +
                        32;   // each of the takes below rounded up to two doubles
   vef_status st = ensure_buffer((void**)&M.work, &M.work_cap, total * sizeof(double));
   if (st != VEF_OK) return st;
@@ -1773,10 +1837,6 @@ static vef_status hrt_run(Mesh& M, const HrtIn& in, double tol, int max_iter, do
   k.cw = reinterpret_cast<double2*>(take(2 * vec));
   k.part = take((size_t)kNumDots * k.ntiles);
   k.st = reinterpret_cast<KState*>(take(sizeof(KState) / sizeof(double)));
-  double* refd = take(refh.size());
-  // pageable source: the copy has taken the data when the call returns
-  VEF_CUDA_TRY(cudaMemcpyAsync(refd, refh.data(), refh.size() * sizeof(double), cudaMemcpyHostToDevice, s));
-  const HrtRef ref{refd, refd + (size_t)S::N * S::NJ};
   HrtOut out{Li, C2, g, f, He, re};
   const size_t smem = sizeof(HrtSmem<P>), ismem = sizeof(HrtInvSmem<P>);
   VEF_CUDA_TRY(cudaFuncSetAttribute(hrt_local_kernel<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
@@ -1786,13 +1846,13 @@ static vef_status hrt_run(Mesh& M, const HrtIn& in, double tol, int max_iter, do
   int dev = 0, sms = 0, inv_per_sm = 0;
   VEF_CUDA_TRY(cudaGetDevice(&dev));
   VEF_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  VEF_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&inv_per_sm, hrt_invert_kernel<P>, 128, ismem));
+  VEF_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&inv_per_sm, hrt_invert_kernel<P>, HrtInvShape<P>::T, ismem));
   {
     KTimer kt(&M, VEF_K_HRT, s);
     hrt_local_kernel<P><<<(unsigned)std::min<long long>(E, (long long)sms * 8), 256, smem, s>>>(
-        E, M.nx, M.ny, tab, ref, in, out, M.dev_status);
-    hrt_invert_kernel<P><<<(unsigned)std::min<long long>(E, (long long)sms * std::max(1, inv_per_sm)), 128, ismem,
-                           s>>>(E, M.nx, M.ny, ref, out, M.dev_status);
+        E, M.nx, M.ny, (M.m + 1) * (M.m + 1), ref, in, out);
+    hrt_invert_kernel<P><<<(unsigned)std::min<long long>(E, (long long)sms * std::max(1, inv_per_sm)),
+                           HrtInvShape<P>::T, ismem, s>>>(E, M.nx, M.ny, ref, out, M.dev_status);
     VEF_CUDA_TRY(cudaGetLastError());
   }
   int it = 0;

@@ -229,6 +229,7 @@ Mesh::~Mesh() {
   cudaFree(nds32);
   cudaFree(dev_status);
   cudaFree(vef_work);
+  cudaFree(hrt_ref);
   cudaFree(bvol);
   cudaFree(work);
   cudaFree(work2);
