@@ -356,25 +356,53 @@ factor_pivot_kernel(long long nmem, const uint32_t* __restrict__ code, const uin
 // rows and beta = 1/r[k] - 1 on the pivot row itself (which turns it into r / r[k]);
 // column k then becomes -A[i][k] / r[k], or 1 / r[k] on the pivot row.  With several rows
 // per lane the reciprocal and the broadcast are shared by RPL rows' FMAs.
+// The columns turn by one place per step (the pivot column is register column 0, the new
+// column goes last), so that the steps run in a loop: unrolled, the elimination is some 60 KB
+// of instructions at p = 3 and 130 KB at p = 4, and warps out of step with one another wait for
+// instruction fetch (256^2 Q3 S12 call: 73.2 ms unrolled, 67.0 ms turned).
 template <int P, typename T> struct ElemShape;
 // EPC elements per CTA: at p = 3 in FP64 a warp holds 8 tasks, and the level-symmetric sets
 // have D = 4 (mod 8) directions for S4 and S12, so one element per CTA would leave half a
 // warp of padding tasks computing; two elements per CTA fill every warp (2 D = 0 mod 8).
-// FP64 is bound by its FP64 pipe, so four rows per lane share each pivot-row broadcast.
+// FP64 is bound by its FP64 pipe, so four rows per lane share each pivot-row broadcast.  NW
+// warps per CTA: the 21 rounds of two elements at S12 over four warps go 6, 5, 5, 5, and the
+// scheduler with six sets the time; in FP64 every CTA is one warp instead (8 per SM by
+// registers), which the SM's four schedulers share evenly (256^2 Q3 S12: 78.0 -> 73.2 ms).
 // FP32 is bound by latency instead (four register-limited warps per scheduler at four rows
 // per lane): two rows per lane halve the registers, so six CTAs fit per SM.
-template <> struct ElemShape<3, double> { static constexpr int RPL = 4, LPU = 4, EPC = 2, MINB = 1; };
-template <> struct ElemShape<3, float> { static constexpr int RPL = 2, LPU = 8, EPC = 4, MINB = 6; };
-template <typename T> struct ElemShape<4, T> { static constexpr int RPL = 2, LPU = 13, EPC = 1, MINB = 1; };
+template <> struct ElemShape<3, double> { static constexpr int RPL = 4, LPU = 4, EPC = 2, NW = 1, MINB = 1; };
+template <> struct ElemShape<3, float> { static constexpr int RPL = 2, LPU = 8, EPC = 4, NW = 4, MINB = 6; };
+template <> struct ElemShape<4, float> { static constexpr int RPL = 2, LPU = 13, EPC = 1, NW = 4, MINB = 1; };
+
+// an element's (or CTA's elements') rounds are spread over `parts` CTAs: CTA blockIdx.x takes
+// [r0, r1)
+__device__ __forceinline__ void part_rounds(int rounds, int parts, int& r0, int& r1) {
+  const int part = blockIdx.x % parts;
+  r0 = (int)((long long)rounds * part / parts);
+  r1 = (int)((long long)rounds * (part + 1) / parts);
+}
+// parts per element group so that single-warp CTAs (8 per SM by registers) come in about
+// kPartWaves waves: with fewer the last wave leaves SMs idle, with more each CTA stages its
+// element for too few rounds.  Whole call without and with parts: 23^2 Q3 S4 0.417 -> 0.313 ms,
+// 64^2 Q3 S6 2.17 -> 2.07, 61 x 47 Q4 S6 5.20 -> 4.70, 64^2 Q4 S12 17.6 -> 16.0; the grids that
+// give six waves by themselves (256^2 Q3 S12) take one part.
+constexpr int kPartWaves = 6;
+static int factor_parts(long long groups, int rounds) {
+  int dev = 0, sms = 1;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const long long want = (long long)sms * 8 * kPartWaves;
+  return (int)std::max(1LL, std::min<long long>(rounds, (want + groups - 1) / groups));
+}
 
 template <int P, typename T, bool Y>
-__global__ void __launch_bounds__(128, ElemShape<P, T>::MINB)
+__global__ void __launch_bounds__(32 * ElemShape<P, T>::NW, ElemShape<P, T>::MINB)
 factor_elem_kernel(int D, long long E, const int* __restrict__ member_of, const uint16_t* __restrict__ finfo,
                    const double* __restrict__ omega, const double* __restrict__ sigma_t,
                    const T* __restrict__ Mm, const T* __restrict__ Gxm, const T* __restrict__ Gym,
                    const T* __restrict__ nds, FaceTab<T> ft, int nx, int ny, long long nmem,
                    T* __restrict__ rec, unsigned int* status, unsigned int* piv_count,
-                   unsigned int* piv_list, int force_pivot, RhsArgs<T> rhs) {
+                   unsigned int* piv_list, int force_pivot, RhsArgs<T> rhs, int parts) {
   constexpr int Q = P + 1, N = Q * Q, NQ = P + 2;
   constexpr int RPL = ElemShape<P, T>::RPL, LPU = ElemShape<P, T>::LPU, UPW = 32 / LPU, EPC = ElemShape<P, T>::EPC;
   constexpr int LD = N + 1;                  // padded shared-memory row stride
@@ -385,8 +413,8 @@ factor_elem_kernel(int D, long long E, const int* __restrict__ member_of, const 
   __shared__ T sN[EPC][4 * NQ * 2];
   __shared__ T sLL[Q][Q][NQ];          // l_a(s_k) l_t(s_k): face basis products
   __shared__ T sW[NQ];                 // face Gauss weights
-  __shared__ T sC[4][UPW][4][NQ];      // per warp and task: w_k Omega . (n ds)_k of each face
-  const long long e0 = (long long)blockIdx.x * EPC;
+  __shared__ T sC[ElemShape<P, T>::NW][UPW][4][NQ];   // per warp and task: w_k Omega . (n ds)_k of each face
+  const long long e0 = (long long)(blockIdx.x / parts) * EPC;
   const int ne = (int)min((long long)EPC, E - e0);   // elements of this CTA
   const int tid = threadIdx.x;
   for (int idx = tid; idx < ne * N * N; idx += blockDim.x) {
@@ -408,12 +436,16 @@ factor_elem_kernel(int D, long long E, const int* __restrict__ member_of, const 
   const int u = lane / LPU, li = lane % LPU, base = u * LPU;
   const int uc = u < UPW ? u : UPW - 1;   // lanes past the last task read a valid slot
   char* recx = (char*)rec + nmem * (long long)L::kStaged;
-  // tasks t = el D + d of the CTA's elements, UPW per warp and round
+  // tasks t = d ne + el of the CTA's elements, UPW per warp and round: a direction's elements
+  // side by side, so that a warp's tasks lie in one quadrant more often (faces no task needs
+  // are skipped)
   const int ntask = ne * D;
-  for (int t0 = warp * UPW; t0 < ntask; t0 += nwarps * UPW) {
+  int r0, r1;   // this CTA's rounds
+  part_rounds((ntask + UPW - 1) / UPW, parts, r0, r1);
+  for (int t0 = (r0 + warp) * UPW; t0 < r1 * UPW; t0 += nwarps * UPW) {
     const int t = t0 + u;
     bool valid = u < UPW && t < ntask;
-    const int tt = valid ? t : 0, el = tt / D, dd = tt % D;
+    const int tt = valid ? t : 0, el = tt % ne, dd = tt / ne;
     const long long e = e0 + el;
     const T mu = (T)omega[2 * dd], eta = (T)omega[2 * dd + 1];
     const uint16_t bits = finfo[(size_t)dd * E + e];
@@ -484,24 +516,27 @@ factor_elem_kernel(int D, long long E, const int* __restrict__ member_of, const 
     }
     bool bad = false;
     // in-place Gauss-Jordan over the task's LPU lanes (no pivoting; the owner of row k
-    // checks its pivot against the row's scale)
+    // checks its pivot against the row's scale).  The columns turn by one place per step: the
+    // pivot column is always the first, the new one goes last, and after N steps every column
+    // is back, so that the steps of one slot share their code
 #pragma unroll
-    for (int k = 0; k < N; ++k) {
-      const int owner = k % LPU, slot = k / LPU;
-      T pr[N];
+    for (int slot = 0; slot < RPL; ++slot) {
+#pragma unroll 1
+      for (int owner = 0; owner < min(LPU, N - slot * LPU); ++owner) {
+        const int k = slot * LPU + owner;
+        T pr[N];
 #pragma unroll
-      for (int j = 0; j < N; ++j) pr[j] = __shfl_sync(FULL, row[slot][j], (base + owner) & 31);
-      if (li == owner) bad = bad || small_pivot<T>(pr[k], scl[slot]);
-      const T inv = pivot_rcp(pr[k]);
+        for (int j = 0; j < N; ++j) pr[j] = __shfl_sync(FULL, row[slot][j], (base + owner) & 31);
+        if (li == owner) bad = bad || small_pivot<T>(pr[0], scl[slot]);
+        const T inv = pivot_rcp(pr[0]);
 #pragma unroll
-      for (int r = 0; r < RPL; ++r) {
-        const int i = li + LPU * r;
-        const T aik = row[r][k];
-        const T beta = (i == k) ? inv - (T)1 : -aik * inv;
+        for (int r = 0; r < RPL; ++r) {
+          const T aik = row[r][0];
+          const T beta = (li + LPU * r == k) ? inv - (T)1 : -aik * inv;
 #pragma unroll
-        for (int j = 0; j < N; ++j)
-          if (j != k) row[r][j] = fma(beta, pr[j], row[r][j]);
-        row[r][k] = (i == k) ? inv : -aik * inv;
+          for (int j = 1; j < N; ++j) row[r][j - 1] = fma(beta, pr[j], row[r][j]);
+          row[r][N - 1] = (li + LPU * r == k) ? inv : -aik * inv;
+        }
       }
     }
     // records: A^{-1} column-major, then the W slots of the interior inflow faces
@@ -597,6 +632,248 @@ factor_elem_kernel(int D, long long E, const int* __restrict__ member_of, const 
     // a task any of whose lanes saw a small pivot goes to the pivoted fallback
     const unsigned bal = __ballot_sync(FULL, bad || force_pivot);
     if (valid && li == 0 && ((bal >> base) & ((1u << LPU) - 1u))) pivot_list_append(piv_count, piv_list, m);
+  }
+}
+
+// The fourth order in FP64.  25 rows fit no whole number of lanes: two tasks of 13 lanes with two
+// rows each leave 22 % of a warp's FP64 lanes without a row.  Here a warp holds five tasks: row
+// i < 24 of task u on lane 6 u + i mod 6, slot i / 6, and the five last rows on lanes 30 (tasks
+// 0..3, one per slot) and 31 (task 4): 125 of 128 slots work.  The rows take 200 registers, so
+// the pivot row is not held: its owner publishes it, with the pivot's reciprocal, through a
+// double buffer in shared memory and every FMA reads its entry there (FP64 issue is slow enough
+// to hide the reads).  One warp per CTA and element.  The operations on each entry and their
+// order are those of factor_elem_kernel, so the records are the same to the last bit.  FP64
+// issue per task falls by a quarter; a 64^2 Q4 S12 call took 22.4 ms with two tasks per warp and
+// takes 16.0, a batch of 16 problems up to 128^2 Q4 S12 125 and 88.6 ms.
+template <bool Y>
+__global__ void __launch_bounds__(32, 8)
+factor_elem4_kernel(int D, long long E, const int* __restrict__ member_of, const uint16_t* __restrict__ finfo,
+                    const double* __restrict__ omega, const double* __restrict__ sigma_t,
+                    const double* __restrict__ Mm, const double* __restrict__ Gxm, const double* __restrict__ Gym,
+                    const double* __restrict__ nds, FaceTab<double> ft, int nx, int ny, long long nmem,
+                    double* __restrict__ rec, unsigned int* status, unsigned int* piv_count,
+                    unsigned int* piv_list, int force_pivot, RhsArgs<double> rhs, int parts) {
+  constexpr int P = 4, Q = P + 1, N = Q * Q, NQ = P + 2, LD = N + 1;
+  constexpr int RPL = 4, LPU = 6, UPW = 5, NB = LPU * RPL;   // NB: rows held by a task's own lanes
+  constexpr unsigned FULL = 0xffffffffu;
+  using L = Rec<P, double>;
+  __shared__ double sM[N * LD], sX[N * LD], sY[N * LD];   // sigma_t M, Gx, Gy
+  __shared__ double sN[4 * NQ * 2];
+  __shared__ double sLL[Q][Q][NQ];      // l_a(s_k) l_t(s_k)
+  __shared__ double sC[UPW][4][NQ];     // per task: w_k Omega . (n ds)_k of each face
+  __shared__ double sRow[2][UPW][LD], sInv[2][UPW];   // pivot row and reciprocal of each task
+  __shared__ double sT[UPW][N];         // per task: Cin of a face, or b
+  __shared__ int sScl[RPL][32];         // largest magnitude of each row as assembled
+  const long long e = blockIdx.x / parts;
+  const int lane = threadIdx.x;
+  for (int idx = lane; idx < N * N; idx += 32) {
+    const int at = (idx / N) * LD + idx % N;
+    const size_t g = (size_t)e * N * N + idx;
+    sM[at] = sigma_t[e] * Mm[g];
+    sX[at] = Gxm[g];
+    sY[at] = Gym[g];
+  }
+  for (int idx = lane; idx < 4 * NQ * 2; idx += 32) sN[idx] = nds[(size_t)e * 4 * NQ * 2 + idx];
+  for (int idx = lane; idx < Q * Q * NQ; idx += 32) {
+    const int qa = idx / (Q * NQ), qt = (idx / NQ) % Q, kk = idx % NQ;
+    sLL[qa][qt][kk] = ft.l[qa][kk] * ft.l[qt][kk];
+  }
+  const bool tail = lane >= UPW * LPU;      // lanes 30, 31
+  const int ul = lane / LPU, li = lane % LPU;
+  // task and row of slot r (lane 31's other slots repeat its first and write nothing)
+  const int task0 = !tail ? ul : lane == 30 ? 0 : UPW - 1, task1 = lane == 30;
+  const int rowb = !tail ? li : NB, row1 = !tail ? LPU : 0;
+  auto task_of = [&](int r) { return task0 + task1 * r; };
+  auto row_of = [&](int r) { return rowb + row1 * r; };
+  auto owns = [&](int r) { return lane < 31 || r == 0; };
+  char* recx = (char*)rec + nmem * (long long)L::kStaged;
+  int r0, r1;
+  part_rounds((D + UPW - 1) / UPW, parts, r0, r1);
+  for (int t0 = r0 * UPW; t0 < r1 * UPW; t0 += UPW) {
+    auto dir = [&](int u) { return min(t0 + u, D - 1); };
+    __syncwarp();
+    for (int idx = lane; idx < UPW * 4 * NQ; idx += 32) {
+      const int u = idx / (4 * NQ), q = idx % (4 * NQ);
+      sC[u][q / NQ][q % NQ] =
+          ft.w[q % NQ] * (omega[2 * dir(u)] * sN[2 * q] + omega[2 * dir(u) + 1] * sN[2 * q + 1]);
+    }
+    __syncwarp();
+    // sigma_t M - mu Gx - eta Gy ...
+    double row[RPL][N];
+#pragma unroll
+    for (int r = 0; r < RPL; ++r) {
+      const int i = row_of(r);
+      const double mu = omega[2 * dir(task_of(r))], eta = omega[2 * dir(task_of(r)) + 1];
+#pragma unroll
+      for (int j = 0; j < N; ++j)
+        row[r][j] = fma(-eta, sY[i * LD + j], fma(-mu, sX[i * LD + j], sM[i * LD + j]));
+    }
+    // ... plus the outflow face terms: row a of task u's face matrix is formed on lane u Q + a
+    // and shuffled to the owner of the face node
+#pragma unroll
+    for (int f = 0; f < 4; ++f) {
+      const int uq = lane < UPW * Q ? lane / Q : UPW - 1, fa = lane % Q;
+      bool out_f = false;
+#pragma unroll
+      for (int k = 0; k < NQ; ++k) out_f = out_f || sC[uq][f][k] > 0.0;
+      if (!__any_sync(FULL, out_f)) continue;
+      double fo[Q];
+#pragma unroll
+      for (int t = 0; t < Q; ++t) fo[t] = 0.0;
+#pragma unroll
+      for (int k = 0; k < NQ; ++k) {
+        const double s = sC[uq][f][k], sp = s > 0.0 ? s : 0.0;
+#pragma unroll
+        for (int t = 0; t < Q; ++t) fo[t] = fma(sp, sLL[fa][t][k], fo[t]);
+      }
+#pragma unroll
+      for (int r = 0; r < RPL; ++r) {
+        const int i = row_of(r), ia = i % Q, ib = i / Q;
+        int pos = -1;
+        if (f == 0 && ib == 0) pos = ia;
+        if (f == 1 && ia == P) pos = ib;
+        if (f == 2 && ib == P) pos = ia;
+        if (f == 3 && ia == 0) pos = ib;
+        if (!__any_sync(FULL, pos >= 0)) continue;
+        const int src = task_of(r) * Q + (pos > 0 ? pos : 0);
+#pragma unroll
+        for (int t = 0; t < Q; ++t) {
+          const double v = __shfl_sync(FULL, fo[t], src);
+          if (pos >= 0) row[r][face_dof<P>(f, t)] += v;
+        }
+      }
+    }
+    // row scales for the pivot guard
+#pragma unroll
+    for (int r = 0; r < RPL; ++r) {
+      int mx = 0;
+#pragma unroll
+      for (int j = 0; j < N; ++j) mx = max(mx, PivotFloor<double>::mag(row[r][j]));
+      sScl[r][lane] = mx;
+    }
+    unsigned bad = 0;   // tasks with a small pivot
+    // in-place Gauss-Jordan, the columns turned by one place per step: the pivot column is
+    // always the first, the new one goes last, and after N steps every column is back
+#pragma unroll 1
+    for (int k = 0; k < N; ++k) {
+      const int b = k & 1;
+      const int ks = k < NB ? k / LPU : -1;   // the slot that holds row k (each its own on the tail lanes)
+      const bool mine = k < NB ? !tail && li == k - ks * LPU : tail;
+#pragma unroll
+      for (int r = 0; r < RPL; ++r) {
+        if (!(ks < 0 || r == ks)) continue;
+        const double inv = pivot_rcp(row[r][0]);
+        if (mine && owns(r)) {
+          const int u = task_of(r);
+          if (small_pivot<double>(row[r][0], sScl[r][lane])) bad |= 1u << u;
+#pragma unroll
+          for (int j = 1; j < N; ++j) sRow[b][u][j] = row[r][j];
+          sInv[b][u] = inv;
+        }
+      }
+      __syncwarp();
+#pragma unroll
+      for (int r = 0; r < RPL; ++r) {
+        const int u = task_of(r);
+        const double inv = sInv[b][u], aik = row[r][0];
+        const bool own = row_of(r) == k;
+        const double beta = own ? inv - 1.0 : -aik * inv;
+        const double* pr = sRow[b][u];
+#pragma unroll
+        for (int j = 1; j < N; ++j) row[r][j - 1] = fma(beta, pr[j], row[r][j]);
+        row[r][N - 1] = own ? inv : -aik * inv;
+      }
+    }
+    // records: A^{-1} column-major ...
+    const int du = t0 + (lane < UPW ? lane : 0);   // lane u < 5 also keeps task u's face data
+    const bool has = lane < UPW && du < D;
+    const uint16_t bits = has ? finfo[(size_t)du * E + e] : 0;
+    auto member = [&](int u) {
+      const long long m = t0 + u < D ? (long long)member_of[(size_t)(t0 + u) * E + e] : -1;
+      return m >= 0 && VEF_IN_RANGE(m, nmem, status) ? m : -1;
+    };
+#pragma unroll
+    for (int r = 0; r < RPL; ++r) {
+      const long long m = owns(r) ? member(task_of(r)) : -1;
+      if (m < 0) continue;
+      double* ai = L::ainv(L::x_at(recx, m)) + row_of(r);
+#pragma unroll
+      for (int j = 0; j < N; ++j) ai[j * N] = row[r][j];
+    }
+    if constexpr (Y) {   // y = A^{-1} b (the sweep's apply, done here)
+#pragma unroll 1
+      for (int r = 0; r < RPL; ++r) {
+        const int u = task_of(r), i = row_of(r), d = t0 + u;
+        if (owns(r))
+          sT[u][i] = d < D ? rhs_b<P, double>(rhs, ft, nds, nx, ny, E, d, (int)e, i, finfo[(size_t)d * E + e],
+                                              omega[2 * d], omega[2 * d + 1])
+                           : 0.0;
+      }
+      __syncwarp();
+#pragma unroll
+      for (int r = 0; r < RPL; ++r) {
+        const int u = task_of(r);
+        double y = 0.0;
+#pragma unroll
+        for (int j = 0; j < N; ++j) y = fma(row[r][j], sT[u][j], y);
+        const long long m = owns(r) ? member(u) : -1;
+        if (m >= 0) rhs.y[(size_t)m * L::kYStride + row_of(r)] = y;
+      }
+    }
+    // ... then the W slots of the interior inflow faces
+    unsigned use[4];
+#pragma unroll
+    for (int f = 0; f < 4; ++f)
+      use[f] = __ballot_sync(FULL, has && (bits & (1u << f)) && nb_elem(nx, ny, (int)e, f) >= 0);
+#pragma unroll
+    for (int f = 0; f < 4; ++f) {
+      if (!use[f]) continue;
+      __syncwarp();
+      // Cin_f[a][t] = sum_k min(c_k, 0) l_a(s_k) l_t(s_k)
+      for (int idx = lane; idx < UPW * N; idx += 32) {
+        const int u = idx / N, q = idx % N;
+        double v = 0.0;
+#pragma unroll
+        for (int k = 0; k < NQ; ++k) {
+          const double s = sC[u][f][k];
+          v = fma(s < 0.0 ? s : 0.0, sLL[q / Q][q % Q][k], v);
+        }
+        sT[u][q] = v;
+      }
+      __syncwarp();
+#pragma unroll
+      for (int r = 0; r < RPL; ++r) {
+        const int u = task_of(r);
+        const long long m = owns(r) && ((use[f] >> u) & 1u) ? member(u) : -1;
+        int slot = 0;
+#pragma unroll
+        for (int g = 0; g < f; ++g) slot += (use[g] >> u) & 1u;
+        double* Wo = m >= 0 ? L::slot(L::s_at(rec, m), L::x_at(recx, m), slot) + row_of(r) : nullptr;
+#pragma unroll
+        for (int t = 0; t < Q; ++t) {
+          double w = 0.0;
+#pragma unroll
+          for (int a = 0; a < Q; ++a) w = fma(row[r][face_dof<P>(f, a)], sT[u][a * Q + t], w);
+          if (m >= 0) Wo[t * N] = w;
+        }
+      }
+    }
+    bad = __reduce_or_sync(FULL, bad);
+    if (has) {
+      const long long m = member(lane);
+      unsigned faces = 0xffffffffu;
+      int n = 0;
+#pragma unroll
+      for (int f = 0; f < 4; ++f)
+        if ((use[f] >> lane) & 1u) {
+          faces = (faces & ~(0xffu << (8 * n))) | ((unsigned)f << (8 * n));
+          ++n;
+        }
+      if (m >= 0) {
+        *reinterpret_cast<uint4*>(L::s_at(rec, m)) = make_uint4((unsigned)e, (unsigned)bits, faces, 0u);
+        if (((bad >> lane) & 1u) || force_pivot) pivot_list_append(piv_count, piv_list, m);
+      }
+    }
   }
 }
 
@@ -1104,13 +1381,22 @@ static vef_status launch_factor(Mesh& M, Schedule& S, const double* sigma_t, boo
   VEF_CUDA_TRY(cudaMemsetAsync(piv_count, 0, sizeof(unsigned int), stream));
   {
   KTimer kt(&M, VEF_K_FACTOR, stream);
-  if constexpr (P >= 3) {
+  if constexpr (P == 4 && sizeof(T) == 8) {
+    auto kern = rhs ? factor_elem4_kernel<true> : factor_elem4_kernel<false>;
+    const int parts = factor_parts(M.E, (S.D + 4) / 5);
+    kern<<<(unsigned)(M.E * parts), 32, 0, stream>>>(S.D, M.E, S.member_of, S.faceinfo, S.omega_dev, sigma_t, Mm, Gx, Gy, nds,
+                                           make_facetab<T>(M.tab), M.nx, M.ny, S.members, (T*)*recp, M.dev_status,
+                                           piv_count, S.pivot_list, force_pivot, ra, parts);
+  } else if constexpr (P >= 3) {
     constexpr int UPW = 32 / ElemShape<P, T>::LPU, EPC = ElemShape<P, T>::EPC;
-    const int warps = std::max(1, std::min(4, (EPC * S.D + UPW - 1) / UPW));
+    constexpr int NW = ElemShape<P, T>::NW;
+    const int rounds = (EPC * S.D + UPW - 1) / UPW, warps = std::max(1, std::min(NW, rounds));
+    const long long groups = (M.E + EPC - 1) / EPC;
+    const int parts = NW == 1 ? factor_parts(groups, rounds) : 1;
     auto kern = rhs ? factor_elem_kernel<P, T, true> : factor_elem_kernel<P, T, false>;
-    kern<<<(unsigned)((M.E + EPC - 1) / EPC), 32 * warps, 0, stream>>>(
+    kern<<<(unsigned)(groups * parts), 32 * warps, 0, stream>>>(
         S.D, M.E, S.member_of, S.faceinfo, S.omega_dev, sigma_t, Mm, Gx, Gy, nds, make_facetab<T>(M.tab),
-        M.nx, M.ny, S.members, (T*)*recp, M.dev_status, piv_count, S.pivot_list, force_pivot, ra);
+        M.nx, M.ny, S.members, (T*)*recp, M.dev_status, piv_count, S.pivot_list, force_pivot, ra, parts);
   } else {
     auto kern = rhs ? factor_kernel<P, T, true> : factor_kernel<P, T, false>;
     kern<<<nblk(S.members, 128), 128, 0, stream>>>(
