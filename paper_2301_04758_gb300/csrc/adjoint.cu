@@ -370,8 +370,9 @@ __device__ __forceinline__ void adj_group_direct(const AdjArgs& a, int d, int s0
 // p+1 values into the slot through which the forward sweep passed the donor's face values;
 // the donor subtracts them from w_d g on its outflow face rows.  Warp 15 streams the
 // singles' records (info + W slots 0, 1), their w_d g rows and slot ids through a ring of
-// chunk buffers (bulk copies); warps 0..11 compute rounds of 12 SPC tasks, the
-// projections summed over a task's rows through a per-warp scratch; warps 12..14 run the
+// chunk buffers (bulk copies); warps 0..11 compute rounds of 12 SPC tasks (r on one lane per
+// row, then through a per-warp scratch one lane or more per projection, whose FMA chain
+// needs no separate products); warps 12..14 run the
 // coupled groups (inner iteration on the transposed blocks); a named barrier separates
 // levels.  Couplings whose slot is missing (receivers in groups, third and fourth W
 // slots, capacity) are read from global memory (slot-id flag bit 1).
@@ -391,7 +392,7 @@ struct AdjShape {
   static constexpr int kRound = kTsOff + CK * 16;
   static constexpr int kMaxRing = 16;
   static constexpr int kBars = 2 * kMaxRing * 8;
-  static constexpr int kScratch = kCompute * SPC * 2 * Q * N * 8;   // per warp [task][slot][t][row]
+  static constexpr int kScratch = kCompute * SPC * N * 8;   // per warp [task][row]: r
   static constexpr int kGs = ((int)sizeof(AdjGroupSmem<P>) + 15) / 16 * 16;
   static constexpr int kGroup = kGroupWarps * kGs;
   static constexpr int kSmemMax = 227 * 1024;
@@ -517,7 +518,10 @@ __global__ void __maxnreg__(128) adjoint_cta_kernel(AdjArgs a) {
   if (ia == P) on_face(1, ib);
   if (ib == P) on_face(2, ia);
   if (ia == 0) on_face(3, ib);
-  double* scratch = scratch_all + (compute ? warp : 0) * (SPC * 2 * Q * N);
+  double* scratch = scratch_all + (compute ? warp : 0) * (SPC * N);
+  // lanes per projection and rows per lane
+  constexpr int PT = 32 / (SPC * 2 * Q) > 0 ? 32 / (SPC * 2 * Q) : 1, NP = (N + PT - 1) / PT;
+  static_assert(SPC * 2 * Q * PT <= 32, "a warp's projections fit its lanes");
   double* radj = a.radj + (size_t)d * a.E * N;
   const int ntr = a.tr_bytes / (Q * (int)sizeof(double));   // trace slots in shared memory
   (void)ntr;
@@ -578,28 +582,38 @@ __global__ void __maxnreg__(128) adjoint_cta_kernel(AdjArgs a) {
               }
             }
             if (VEF_IN_RANGE(e, a.E, a.status)) radj[(size_t)e * N + i] = r;
-            // this task's projections onto its donors' faces, W slots 0 and 1 (zero slots
-            // of absent faces give zero products)
-            const double* W = L::slot(rs, nullptr, 0);
-#pragma unroll
-            for (int sl = 0; sl < 2; ++sl)
-#pragma unroll
-              for (int t = 0; t < Q; ++t)
-                scratch[((s_lane * 2 + sl) * Q + t) * N + i] = W[sl * L::kSlot + t * N + i] * r;
+            scratch[s_lane * N + i] = r;
           }
           __syncwarp();
-          for (int q = lane; !failed && q < SPC * 2 * Q; q += 32) {
+          // the tasks' projections onto their donors' faces, s_t = sum_i W[t][i] r_i for W slots
+          // 0 and 1: one FMA chain per (task, slot, t) and part of the rows
+          {
+            const int q = lane / PT, part = lane % PT;
             const int s = q / (2 * Q), sl = (q / Q) % 2, t = q % Q;
             const int tks = tk0 + warp * SPC + s;
-            if (tks >= cend) continue;
-            const uint4 tss = *reinterpret_cast<const uint4*>(rb + Sh::kTsOff + tks * 16);
-            const unsigned wid = (tss.x >> (16 * sl)) & 0xffffu;
-            if (wid == kTraceZero || !VEF_IN_RANGE(wid, ntr, a.status)) continue;
-            const double* pr = scratch + ((s * 2 + sl) * Q + t) * N;
+            const bool on = !failed && q < SPC * 2 * Q && tks < cend;
             double sum = 0.0;
+            unsigned wid = kTraceZero;
+            if (on) {
+              const uint4 tss = *reinterpret_cast<const uint4*>(rb + Sh::kTsOff + tks * 16);
+              wid = (tss.x >> (16 * sl)) & 0xffffu;
+              const double* W = L::slot((const char*)rb + tks * L::kStaged, nullptr, 0) + sl * L::kSlot + t * N;
+              const double* rv = scratch + s * N;
 #pragma unroll
-            for (int j = 0; j < N; ++j) sum += pr[j];
-            tr[wid * Q + t] = sum;
+              for (int jj = 0; jj < NP; ++jj) {
+                // columns of W lie 2^p' words apart at p = 1 and 3: each lane starts at another
+                // row, so that a warp's reads fall into different banks
+                const int j = part * NP + (P == 3 ? (jj + q) % NP : P == 1 ? (jj + q / 4) % NP : jj);
+                if (N % PT == 0 || j < N) sum = fma(W[j], rv[j], sum);
+              }
+            }
+            if constexpr (PT > 1) {
+              double all = sum;
+#pragma unroll
+              for (int o = 1; o < PT; ++o) all += __shfl_down_sync(FULL, sum, o);
+              sum = all;
+            }
+            if (on && part == 0 && wid != kTraceZero && VEF_IN_RANGE(wid, ntr, a.status)) tr[wid * Q + t] = sum;
           }
           __syncwarp();
         }
