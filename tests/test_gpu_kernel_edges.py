@@ -1,10 +1,11 @@
-"""Edges of the dispatch of the element factorisation and the hybridized VEF solve: remainders
-of the tasks per warp and the elements per CTA, pivot fallbacks, tiles wider than a CTA."""
+"""Edges of the dispatch of the element factorisation, the mixed path's first residual and the
+hybridized VEF solve: remainders of the tasks per warp and the elements per CTA, boundary
+data, pivot fallbacks, tiles wider than a CTA."""
 import numpy as np
 import pytest
 
 from _gpu import dev, host, rel, random_problem
-from oracle.transport import Discretization, sweep as o_sweep
+from oracle.transport import Discretization, sweep as o_sweep, residual_terms
 
 pytestmark = pytest.mark.gpu
 
@@ -39,6 +40,28 @@ def test_factorisation_with_partial_warps_and_ctas(lib, p, nx, ny, sn, D):
     assert rel(host(psi), ref) < 1e-12, info
     psi, info = _sweep(prob, precision="mixed")
     assert rel(host(psi), ref) < 1e-10, info
+
+
+@pytest.mark.parametrize("p", [1, 2, 3, 4])
+@pytest.mark.parametrize("aniso,inflow", [(False, False), (True, True)])
+def test_first_residual_of_the_mixed_path(lib, p, aniso, inflow):
+    """With one fixed pass psi is the FP32 sweep's result; with two, info.rel_residual is
+    ||r|| / ||b|| at that iterate.  The library forms r to about 2^-46 of the terms it sums
+    (FP32 pairs) or better, so the ratio agrees with the oracle's element-by-element residual of
+    the same psi to 2^-44 of the size of its terms."""
+    nx, ny, sn = 9, 7, 6
+    prob = random_problem(nx, ny, 3, 0.08, p, sn, seed=720 + p, aniso=aniso, with_inflow=inflow)
+    disc = Discretization(nx, ny, 3, 0.08, p)
+    args = (disc, prob["omega"], prob["sigma_t"], prob["sigma_s"])
+    data = dict(phi_in=prob["phi_in"], source=prob["source"], inflow=prob["inflow"])
+    psi0, _ = _sweep(prob, precision="mixed", tol=-1.0, max_passes=1)
+    psi0 = host(psi0)
+    assert np.array_equal(psi0, psi0.astype(np.float32).astype(np.float64))
+    r, size = residual_terms(*args, psi0, **data)
+    b, _ = residual_terms(*args, np.zeros_like(psi0), **data)
+    _, info = _sweep(prob, precision="mixed", tol=-1.0, max_passes=2)
+    tol = 2.0 ** -44 * np.linalg.norm(size) / np.linalg.norm(r)
+    assert abs(info["rel_residual"] / (np.linalg.norm(r) / np.linalg.norm(b)) - 1.0) < tol, (info, tol)
 
 
 def _vef_case(nx, ny, p, seed):
