@@ -372,7 +372,7 @@ __device__ __forceinline__ void adj_group_direct(const AdjArgs& a, int d, int s0
 // singles' records (info + W slots 0, 1), their w_d g rows and slot ids through a ring of
 // chunk buffers (bulk copies); warps 0..11 compute rounds of 12 SPC tasks (r on one lane per
 // row, then through a per-warp scratch one lane or more per projection, whose FMA chain
-// needs no separate products); warps 12..14 run the
+// needs no separate products: 128^2 Q2 S8 flux and gradients 7.87 -> 7.60 ms); warps 12..14 run the
 // coupled groups (inner iteration on the transposed blocks); a named barrier separates
 // levels.  Couplings whose slot is missing (receivers in groups, third and fourth W
 // slots, capacity) are read from global memory (slot-id flag bit 1).

@@ -1048,9 +1048,13 @@ assemble64_thread_kernel(long long nmem, const uint32_t* __restrict__ code, cons
 // internal upwind traces as unknowns) reduced to its interface.  One CTA per group forms
 // I + R in shared memory and inverts it in place (Gauss-Jordan with partial pivoting, in
 // FP64); the inverse is stored column-major.  Trace unknowns are numbered by member, then
-// face, then face node; the sweep numbers them the same way.
+// face, then face node; the sweep numbers them the same way.  The largest groups set the time
+// (one CTA's FP64 pipe and a chain of steps), so they start first and a step has two barriers:
+// whole calls 200^2 Q1 S16 5.63 -> 5.57 ms, 61 x 47 Q4 S6 4.70 -> 4.55, 64^2 Q3 S6 2.07 -> 2.01
+// against five barriers, 128 threads and ascending order.
+constexpr int kGroupThreads = 256;
 template <int P, typename T>
-__global__ void __launch_bounds__(128)
+__global__ void __launch_bounds__(kGroupThreads)
 group_factor_kernel(int g0, const int* __restrict__ grp_slot, const int* __restrict__ grp_nt,
                     const long long* __restrict__ grp_toff, const int* __restrict__ slot_first,
                     const int* __restrict__ slot_count, const uint32_t* __restrict__ member_nbpos,
@@ -1063,9 +1067,10 @@ group_factor_kernel(int g0, const int* __restrict__ grp_slot, const int* __restr
   extern __shared__ __align__(16) double gsm[];
   __shared__ uint32_t cpl[NC];
   __shared__ int perm[kGroupMaxTrace];
-  __shared__ double colk[kGroupMaxTrace];
-  __shared__ int piv_row, ncpl;
-  const int g = g0 + (int)blockIdx.x, tid = threadIdx.x, nth = blockDim.x;
+  __shared__ double colk[kGroupMaxTrace], prow[kGroupMaxTrace], krow[kGroupMaxTrace];
+  __shared__ int ncpl;
+  // groups are numbered by size: the largest first
+  const int g = g0 + (int)(gridDim.x - 1 - blockIdx.x), tid = threadIdx.x, nth = blockDim.x;
   const int sl = grp_slot[g], nt = grp_nt[g];
   const int first = slot_first[sl], m = slot_count[sl];
   const char* recx = (const char*)rec + nmem * (long long)L::kStaged;
@@ -1105,46 +1110,41 @@ group_factor_kernel(int g0, const int* __restrict__ grp_slot, const int* __restr
       Mx[r * nt + col] = v;
     }
   }
+  // two barriers per step: every warp finds the pivot row itself (by the bit patterns of the
+  // magnitudes, which order like the numbers: no FP64 comparisons); the scaled pivot row, the
+  // row it changes places with and the pivot column go to buffers, from which each warp updates
+  // its own rows
   for (int k = 0; k < nt; ++k) {
     __syncthreads();
-    if (tid < 32) {   // pivot: largest |entry| of column k on or below the diagonal
-      double best = -1.0;
-      int bi = k;
-      for (int i = k + tid; i < nt; i += 32) {
-        const double v = fabs(Mx[i * nt + k]);
-        if (v > best) { best = v; bi = i; }
-      }
+    long long best = -1;
+    int pr = k;
+    for (int i = k + lane; i < nt; i += 32) {
+      const long long v = __double_as_longlong(Mx[i * nt + k]) & 0x7fffffffffffffffLL;
+      if (v > best && v <= 0x7ff0000000000000LL) { best = v; pr = i; }   // (not a NaN)
+    }
 #pragma unroll
-      for (int off = 16; off > 0; off >>= 1) {
-        const double ob = __shfl_down_sync(0xffffffffu, best, off);
-        const int oi = __shfl_down_sync(0xffffffffu, bi, off);
-        if (ob > best || (ob == best && oi < bi)) { best = ob; bi = oi; }
-      }
-      if (tid == 0) {
-        piv_row = bi;
-        perm[k] = bi;
-        if (!(best > 1e-300)) atomicOr(status, kDevSingular);
-      }
+    for (int off = 16; off > 0; off >>= 1) {
+      const long long ob = __shfl_xor_sync(0xffffffffu, best, off);
+      const int oi = __shfl_xor_sync(0xffffffffu, pr, off);
+      if (ob > best || (ob == best && oi < pr)) { best = ob; pr = oi; }
+    }
+    if (tid == 0) {
+      perm[k] = pr;
+      if (best < 0 || !(__longlong_as_double(best) > 1e-300)) atomicOr(status, kDevSingular);
+    }
+    const double inv = 1.0 / Mx[pr * nt + k];
+    for (int j = tid; j < nt; j += nth) {
+      prow[j] = j == k ? inv : Mx[pr * nt + j] * inv;
+      krow[j] = Mx[k * nt + j];
+      colk[j] = j == pr ? Mx[k * nt + k] : Mx[j * nt + k];
     }
     __syncthreads();
-    const int pr = piv_row;
-    if (pr != k)
-      for (int j = tid; j < nt; j += nth) {
-        const double t = Mx[k * nt + j];
-        Mx[k * nt + j] = Mx[pr * nt + j];
-        Mx[pr * nt + j] = t;
-      }
-    __syncthreads();
-    const double inv = 1.0 / Mx[k * nt + k];
-    for (int i = tid; i < nt; i += nth) colk[i] = Mx[i * nt + k];
-    __syncthreads();
-    for (int j = tid; j < nt; j += nth) Mx[k * nt + j] = j == k ? inv : Mx[k * nt + j] * inv;
-    __syncthreads();
     for (int i = wid; i < nt; i += nw) {
-      if (i == k) continue;
       const double ci = colk[i];
+      double* Mi = Mx + i * nt;
+      const double* old = i == pr ? krow : Mi;
       for (int j = lane; j < nt; j += 32)
-        Mx[i * nt + j] = j == k ? -ci * inv : fma(-ci, Mx[k * nt + j], Mx[i * nt + j]);
+        Mi[j] = i == k ? prow[j] : j == k ? -ci * inv : fma(-ci, prow[j], old[j]);
     }
   }
   // undo the row interchanges as column interchanges, last first
@@ -1314,7 +1314,7 @@ static vef_status launch_group_factor(Schedule& S, const void* rec, cudaStream_t
     const size_t smem = (size_t)S.max_nt * S.max_nt * sizeof(double);
     VEF_CUDA_TRY(cudaFuncSetAttribute(group_factor_kernel<P, T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       (int)smem));
-    group_factor_kernel<P, T><<<(unsigned)(S.ngroups - up[2]), 128, smem, stream>>>(
+    group_factor_kernel<P, T><<<(unsigned)(S.ngroups - up[2]), kGroupThreads, smem, stream>>>(
         (int)up[2], S.grp_slot, S.grp_nt, S.grp_toff, S.slot_first, S.slot_count, S.member_nbpos,
         (const T*)rec, S.members, (T*)*gp, status);
     VEF_CUDA_TRY(cudaGetLastError());
