@@ -188,10 +188,6 @@ def bytes_moments(p, D, nq2=None):
 HBM_MEASURED = "MEASURED_PEAKS.json hbm_gbs (measured)"
 HBM_FALLBACK = "fallback: 6.8 TB/s, an earlier GB300 copy measurement (MEASURED_PEAKS.json absent)"
 FP64_SRC = "derived: 152 SM x 2 FP64 FMA/clk x 2 flop x 2070 MHz"
-# the first residual of a mixed inversion at p >= 3 is formed in compensated FP32 pairs, twelve
-# FP32 operations per multiply-add
-PAIR_PEAK_GFLOPS = 152 * 128 * 2 * 2.070 / 12
-PAIR_SRC = "derived: 152 SM x 128 FP32 operations/clk / 12 per compensated FMA x 2 flop x 2070 MHz"
 FP32_SRC = "derived: 152 SM x 128 FP32 FMA/clk x 2 flop x 2070 MHz"
 
 
@@ -384,8 +380,7 @@ def roofline_report(prof64, prof32, p, D, E, steps, K, hbm_gbs, fp64_meas_gflops
                         bytes_sweep(p, word=4) + bytes_apply(p, D, word=4) * (corr if fused else 1.0)
                         + corr * 8.0 * n * (1 - 1 / D),
                         FP32_PEAK_GFLOPS, FP32_SRC),
-              "residual": res + ((FP64_PEAK_GFLOPS, FP64_SRC) if residual_stored or p < 3
-                                 else (PAIR_PEAK_GFLOPS, PAIR_SRC)),
+              "residual": res + (FP64_PEAK_GFLOPS, FP64_SRC),
               "moments": (flops_moments(p, D), bytes_moments(p, D), FP64_PEAK_GFLOPS, FP64_SRC)}
     roof32 = roofline_entries(prof32, work32, E * D, hbm_gbs, hbm_src)
     roofline32 = dominant_roofline(prof32, roof32, lambda k: None)

@@ -155,7 +155,6 @@ struct Mesh {
   float* Gx32 = nullptr;
   float* Gy32 = nullptr;
   float* nds32 = nullptr;
-  double* one = nullptr;    // [E][3][n] the element operator's parts on a constant (with the FP32 copies)
   std::vector<double> nds_host;  // host copy for schedule building
   double* ctrl_dev = nullptr;    // [E][(m+1)^2][2] control points
   std::shared_ptr<void> map_tab; // mesh-order Lagrange tables (MapTab, mesh.cu)
@@ -192,8 +191,6 @@ class KTimer {
 };
 
 vef_status ensure_buffer(void** ptr, size_t* cap, size_t bytes);
-// the lowest order whose first residual of the mixed path is formed in FP32 pairs
-constexpr int kPairMinP = 3;
 vef_status mesh_float_copies(Mesh* mesh, cudaStream_t stream);
 // Right-hand side of a single transport inversion, applied by the factorisation itself:
 // y = A^{-1} b for every task, written in schedule order into the mesh's y buffer, so the

@@ -197,36 +197,7 @@ vef_status ensure_buffer(void** ptr, size_t* cap, size_t bytes) {
   return VEF_OK;
 }
 
-// What the FP64 residual in FP32 pairs takes apart from a constant: per element and row the row
-// sums of M, and of Gx and Gy less the face terms of a constant over the whole boundary
-// ([E][3][n]; the latter two vanish but for quadrature).
-__global__ void one_kernel(long long E, int p, int n, int nq, Tab1D tab, const double* __restrict__ M,
-                           const double* __restrict__ Gx, const double* __restrict__ Gy,
-                           const double* __restrict__ nds, double* __restrict__ one) {
-  const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (t >= E * 3 * n) return;
-  const long long e = t / (3 * n);
-  const int c = (int)(t / n % 3), i = (int)(t % n), q = p + 1, xa = i % q, xb = i / q;
-  const double* row = (c == 0 ? M : c == 1 ? Gx : Gy) + (e * n + i) * n;
-  double v = 0.0;
-  for (int j = 0; j < n; ++j) v += row[j];
-  for (int f = 0; f < 4 && c > 0; ++f) {
-    const int pos = f == 0 ? (xb == 0 ? xa : -1) : f == 1 ? (xa == p ? xb : -1)
-                  : f == 2 ? (xb == p ? xa : -1) : (xa == 0 ? xb : -1);
-    for (int k = 0; k < nq && pos >= 0; ++k)
-      v -= tab.glw[k] * nds[((e * 4 + f) * nq + k) * 2 + c - 1] * tab.l[pos][k];
-  }
-  one[t] = v;
-}
-
 vef_status mesh_float_copies(Mesh* mesh, cudaStream_t stream) {
-  if (mesh->p >= kPairMinP && !mesh->one) {
-    const long long n1 = mesh->E * 3 * mesh->n;
-    VEF_CUDA_TRY(cudaMalloc(&mesh->one, n1 * sizeof(double)));
-    one_kernel<<<blocks_for(n1, 256), 256, 0, stream>>>(mesh->E, mesh->p, mesh->n, mesh->nq, mesh->tab, mesh->Mmat,
-                                                        mesh->Gx, mesh->Gy, mesh->nds, mesh->one);
-    VEF_CUDA_TRY(cudaGetLastError());
-  }
   if (mesh->Mmat32) return VEF_OK;
   const long long nn = mesh->E * mesh->n * mesh->n;
   const long long nf = mesh->E * 4 * mesh->nq * 2;
@@ -256,7 +227,6 @@ Mesh::~Mesh() {
   cudaFree(Gx32);
   cudaFree(Gy32);
   cudaFree(nds32);
-  cudaFree(one);
   cudaFree(dev_status);
   cudaFree(vef_work);
   cudaFree(hrt_ref);

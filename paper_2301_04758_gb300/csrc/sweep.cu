@@ -1264,262 +1264,6 @@ residual_mf_kernel(int D, long long E, int nx, int ny, long long nbf, const doub
   }
 }
 
-// Unevaluated sums of two FP32 numbers (48 to 49 bits), in the arithmetic of Dekker (1971) and
-// the compensated dot product of Ogita, Rump and Oishi (2005): GB300 issues 64 FP32
-// multiply-adds for one in FP64, so a term at eleven FP32 operations is six times cheaper than
-// at one FP64 operation.  The intrinsics keep the compiler from contracting across the steps.
-struct Pair { float h, l; };
-__device__ __forceinline__ Pair pair_split(double x) {
-  const float h = (float)x;
-  return {h, (float)(x - (double)h)};
-}
-// s + c += p + e, the rounding error of s + p (two-sum) and e going to c
-__device__ __forceinline__ void pair_add(Pair& a, float p, float e) {
-  const float t = __fadd_rn(a.h, p), z = __fsub_rn(t, a.h);
-  const float err = __fadd_rn(__fsub_rn(a.h, __fsub_rn(t, z)), __fsub_rn(p, z));
-  a.l = __fadd_rn(a.l, __fadd_rn(err, e));
-  a.h = t;
-}
-// a += m x
-__device__ __forceinline__ void pair_fma(Pair& a, float mh, float ml, Pair x) {
-  const float p = __fmul_rn(mh, x.h);
-  pair_add(a, p, fmaf(ml, x.h, fmaf(mh, x.l, fmaf(mh, x.h, -p))));
-}
-// a - b, exact
-__device__ __forceinline__ Pair pair_diff(float a, float b) {
-  const float s = __fsub_rn(a, b), z = __fsub_rn(s, a);
-  return {s, __fsub_rn(__fsub_rn(a, __fsub_rn(s, z)), __fadd_rn(b, z))};
-}
-__device__ __forceinline__ Pair pair_mul(Pair a, Pair b) {
-  const float p = __fmul_rn(a.h, b.h);
-  return {p, fmaf(a.l, b.h, fmaf(a.h, b.l, fmaf(a.h, b.h, -p)))};
-}
-
-// The same residual for an iterate x that holds FP32 values (the result of the first FP32
-// sweep), with the element operator applied in FP32 pairs to the differences d = x - x_c from
-// the value x_c at one of the element's nodes:
-//     L x = L d + x_c (L 1),  (L 1)_i = sigma_t sum_j M_ij - mu sx_i - eta sy_i,
-// sx_i = sum_j Gx_ij minus row i of the face terms of a constant over the whole boundary
-// (zero but for quadrature).  The pair products carry 2^-47 of their terms; on d the
-// terms are those that vary over the element, so r comes out nearly as in FP64 and the
-// result's error does not grow (psi against the FP64 path at two fixed passes: 1.314e-13 to
-// 1.324e-13 on 40 x 33 Q3 S8, the largest entry 7.7e-13 to 7.4e-13; 2.081e-13 to 2.082e-13 at
-// Q4; on x itself 1.356e-13 and 2.115e-13).  x_c (L 1), b, the difference and the norms are
-// FP64.  5.8 ms at 256^2 Q3 S12 with the apply, where the FP64 form takes 13.7 (FP64 issue), a
-// whole call 26.2 -> 17.6.  p <= 2 keep the FP64 form: a call there would gain a tenth, with
-// errors 1 to 2 % larger on 40 x 33.  Layout
-// as in residual_mf_kernel; M, Gx, Gy, the face normals (times the Gauss weights), the face
-// basis and the directions are split once per element or CTA.
-template <int P, bool FY>
-__global__ void __launch_bounds__(128)
-residual_pair_kernel(int D, long long E, int nx, int ny, long long nbf, const double* __restrict__ omega,
-                     const double* __restrict__ sigma_t, const double* __restrict__ Mm,
-                     const double* __restrict__ Gxm, const double* __restrict__ Gym,
-                     const double* __restrict__ nds, const double* __restrict__ one,
-                     const double* __restrict__ bvol,
-                     const double* __restrict__ src_aniso, const double* __restrict__ inflow,
-                     const float* __restrict__ x, FaceTab<double> ft, double* __restrict__ r,
-                     double* __restrict__ norms, const int* __restrict__ member_of,
-                     const float* __restrict__ recx32, float* __restrict__ y32, long long nmem,
-                     unsigned int* status) {
-  constexpr int Q = P + 1, N = Q * Q, NQ = P + 2, LD = N + 1;
-  constexpr int UPW = 32 / N, NPT = 4 * NQ, ROUNDS = (NPT + N - 1) / N;
-  constexpr int GZ = NPT;                   // a zero block after the face points
-  extern __shared__ float4 sOm[];           // [D] the directions as pairs
-  __shared__ float2 sM[N * LD], sX[N * LD], sY[N * LD];
-  __shared__ float4 sN[NPT];                // w_k (n ds)_k as pairs
-  __shared__ float2 sL[Q][NQ];              // l_t(s_k)
-  __shared__ float2 sP[4][UPW][N];          // d of each warp's tasks
-  __shared__ float2 sG[4][UPW][NPT + NQ];   // c_k psi_hat at the face points, then zeros
-  __shared__ double sB[4][UPW][NPT + NQ];   // c_k psi_bar at boundary inflow points (for ||b||)
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
-  const int u = lane / N, li = lane % N;
-  const int uc = u < UPW ? u : UPW - 1;
-  // the faces row li lies on: offsets of their points in sG and the node position on each
-  const int ia = li % Q, ib = li / Q;
-  int oA = GZ, pA = 0, oB = GZ, pB = 0;
-  {
-    int nf = 0;
-    auto on = [&](int f, int pos) {
-      if (nf++ == 0) { oA = f * NQ; pA = pos; } else { oB = f * NQ; pB = pos; }
-    };
-    if (ib == 0) on(0, ia);
-    if (ia == P) on(1, ib);
-    if (ib == P) on(2, ia);
-    if (ia == 0) on(3, ib);
-  }
-  for (int d = tid; d < D; d += blockDim.x) {
-    const Pair a = pair_split(omega[2 * d]), b = pair_split(omega[2 * d + 1]);
-    sOm[d] = make_float4(a.h, a.l, b.h, b.l);
-  }
-  for (int idx = tid; idx < Q * NQ; idx += blockDim.x) {
-    const Pair a = pair_split(ft.l[idx / NQ][idx % NQ]);
-    sL[idx / NQ][idx % NQ] = make_float2(a.h, a.l);
-  }
-  if (u < UPW)
-    for (int k = li; k < NQ; k += N) {
-      sG[warp][u][GZ + k] = make_float2(0.0f, 0.0f);
-      sB[warp][u][GZ + k] = 0.0;
-    }
-  double rr = 0.0, bb = 0.0;
-  for (long long e = blockIdx.x; e < E; e += gridDim.x) {
-    __syncthreads();   // the previous element's tables are no longer read
-    for (int idx = tid; idx < N * N; idx += blockDim.x) {
-      const int at = (idx / N) * LD + idx % N;
-      const size_t g = (size_t)e * N * N + idx;
-      const Pair m = pair_split(Mm[g]), gx = pair_split(Gxm[g]), gy = pair_split(Gym[g]);
-      sM[at] = make_float2(m.h, m.l);
-      sX[at] = make_float2(gx.h, gx.l);
-      sY[at] = make_float2(gy.h, gy.l);
-    }
-    for (int q = tid; q < NPT; q += blockDim.x) {
-      const double* v = nds + ((size_t)e * NPT + q) * 2;
-      const Pair a = pair_split(ft.w[q % NQ] * v[0]), b = pair_split(ft.w[q % NQ] * v[1]);
-      sN[q] = make_float4(a.h, a.l, b.h, b.l);
-    }
-    __syncthreads();
-    const double* one_e = one + (size_t)e * 3 * N;
-    const double st64 = sigma_t[e], one_m = st64 * one_e[li], one_x = one_e[N + li], one_y = one_e[2 * N + li];
-    const Pair st = pair_split(st64);
-    const int ie = (int)(e % nx), je = (int)(e / nx);
-    const bool bnd = inflow && (ie == 0 || je == 0 || ie == nx - 1 || je == ny - 1);
-    const double bv = bvol[(size_t)e * N + li];
-    for (int d0 = warp * UPW; d0 < D; d0 += nwarps * UPW) {
-      const int d = d0 + u;
-      const bool valid = u < UPW && d < D;
-      const int dd = valid ? d : 0;
-      const float4 om = sOm[dd];
-      const size_t rowbase = ((size_t)dd * E + e) * N;
-      const float xi = valid ? x[rowbase + li] : 0.0f;
-      const float xc = __shfl_sync(0xffffffffu, xi, uc * N + (P / 2) * (Q + 1));
-      __syncwarp();
-      if (u < UPW) {
-        const Pair dx = pair_diff(xi, xc);
-        sP[warp][u][li] = make_float2(dx.h, dx.l);
-      }
-      __syncwarp();
-      // face points: c_k psi_hat as in residual_mf_kernel, less c_k x_c
-#pragma unroll
-      for (int rd = 0; rd < ROUNDS; ++rd) {
-        const int q = li + N * rd;
-        if (u < UPW && q < NPT) {
-          const int f = q / NQ, k = q % NQ;
-          const float4 nn = sN[q];
-          Pair c = pair_mul({om.x, om.y}, {nn.x, nn.y});
-          pair_fma(c, om.z, om.w, Pair{nn.z, nn.w});
-          const float ch = __fadd_rn(c.h, c.l);
-          c.l = __fadd_rn(__fsub_rn(c.h, ch), c.l);
-          c.h = ch;
-          const int nb = nb_elem(nx, ny, (int)e, f);
-          const bool own = c.h >= 0.0f;
-          Pair g = {0.0f, 0.0f};
-          double tb = 0.0;
-          if (own) {
-#pragma unroll
-            for (int t = 0; t < Q; ++t) {
-              const float2 lt = sL[t][k], dx = sP[warp][u][face_dof<P>(f, t)];
-              pair_fma(g, lt.x, lt.y, Pair{dx.x, dx.y});
-            }
-          } else if (nb >= 0) {
-            const float* src = x + ((size_t)dd * E + nb) * N;
-#pragma unroll
-            for (int t = 0; t < Q; ++t) {
-              const float2 lt = sL[t][k];
-              pair_fma(g, lt.x, lt.y, pair_diff(src[face_dof<P>((f + 2) & 3, t)], xc));
-            }
-          } else if (inflow) {
-            const double pb = inflow[((size_t)dd * nbf + bface(nx, ny, (int)e, f)) * NQ + k];
-            tb = ((double)c.h + (double)c.l) * pb;
-            g = pair_split(pb - (double)xc);
-          } else {
-            g.h = -xc;
-          }
-          g = pair_mul(c, g);
-          sG[warp][u][q] = make_float2(g.h, g.l);
-          if (bnd) sB[warp][u][q] = tb;
-        }
-      }
-      // volume part, row li
-      Pair am = {0.0f, 0.0f}, ax = am, ay = am;
-#pragma unroll
-      for (int j = 0; j < N; ++j) {
-        const float2 dx = sP[warp][uc][j];
-        const Pair xj = {dx.x, dx.y};
-        const float2 m = sM[li * LD + j], gx = sX[li * LD + j], gy = sY[li * LD + j];
-        pair_fma(am, m.x, m.y, xj);
-        pair_fma(ax, gx.x, gx.y, xj);
-        pair_fma(ay, gy.x, gy.y, xj);
-      }
-      Pair lx = pair_mul(st, am);   // L d, row li
-      pair_fma(lx, -om.x, -om.y, ax);
-      pair_fma(lx, -om.z, -om.w, ay);
-      double b = bv;
-      if (src_aniso) {
-        const double* qd = src_aniso + rowbase;
-        const double* Me = Mm + ((size_t)e * N + li) * N;
-#pragma unroll
-        for (int j = 0; j < N; ++j) b = fma(Me[j], qd[j], b);
-      }
-      __syncwarp();
-#pragma unroll
-      for (int k = 0; k < NQ; ++k) {
-        const float2 ga = sG[warp][uc][oA + k], gb = sG[warp][uc][oB + k], la = sL[pA][k], lb = sL[pB][k];
-        pair_fma(lx, la.x, la.y, Pair{ga.x, ga.y});
-        pair_fma(lx, lb.x, lb.y, Pair{gb.x, gb.y});
-      }
-      double bs = 0.0;
-      if (bnd) {
-#pragma unroll
-        for (int k = 0; k < NQ; ++k) {
-          bs = fma(sB[warp][uc][oA + k], ft.l[pA][k], bs);
-          bs = fma(sB[warp][uc][oB + k], ft.l[pB][k], bs);
-        }
-      }
-      const double l1 = fma(-omega[2 * dd + 1], one_y, fma(-omega[2 * dd], one_x, one_m));
-      const double ri = (fma(-(double)xc, l1, b) - (double)lx.h) - (double)lx.l;
-      if (valid) {
-        r[rowbase + li] = ri;
-        rr = fma(ri, ri, rr);
-        bb = fma(b - bs, b - bs, bb);
-      }
-      if constexpr (FY) {
-        using L = Rec<P, float>;
-        const long long m = valid ? (long long)member_of[(size_t)dd * E + e] : 0;
-        const bool ok = valid && VEF_IN_RANGE(m, nmem, status);
-        const float rf = ok ? (float)ri : 0.0f;
-        const float* ai = L::ainv(L::x_at(recx32, ok ? m : 0));
-        float y = 0.0f;
-#pragma unroll
-        for (int j = 0; j < N; ++j) {
-          const float bj = __shfl_sync(0xffffffffu, rf, (uc * N + j) & 31);
-          if (ok) y += ai[j * N + li] * bj;
-        }
-        if (ok) y32[(size_t)m * L::kYStride + li] = y;
-      }
-    }
-  }
-  __shared__ double red[2][32];
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) {
-    rr += __shfl_xor_sync(0xffffffffu, rr, off);
-    bb += __shfl_xor_sync(0xffffffffu, bb, off);
-  }
-  if (lane == 0) {
-    red[0][warp] = rr;
-    red[1][warp] = bb;
-  }
-  __syncthreads();
-  if (tid == 0) {
-    double sr = 0.0, sb = 0.0;
-    for (int w = 0; w < nwarps; ++w) {
-      sr += red[0][w];
-      sb += red[1][w];
-    }
-    atomicAdd(norms, sr);
-    atomicAdd(norms + 1, sb);
-  }
-}
-
 __global__ void cast_add_kernel(long long n, const float* __restrict__ delta, double* __restrict__ psi,
                                 int accumulate) {
   long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
@@ -1796,10 +1540,9 @@ static vef_status launch_sweep(const SweepCall& c0, const double* rhs, T* out) {
 
 // The FP64 residual of the mixed defect correction.  With form_y (matrix-free form only) it
 // also writes the FP32 correction sweep's y = A^{-1} r, so that sweep skips its apply.
-// x32: the iterate as FP32 values where psi holds just those (after the first sweep), or null
 template <int P>
-static vef_status launch_residual(const SweepCall& c, const double* psi, const float* x32, double* r,
-                                  double* norms, bool form_y = false) {
+static vef_status launch_residual(const SweepCall& c, const double* psi, double* r, double* norms,
+                                  bool form_y = false) {
   Mesh& M = *c.mesh;
   Schedule& S = *c.S;
   constexpr int N = (P + 1) * (P + 1);
@@ -1818,22 +1561,6 @@ static vef_status launch_residual(const SweepCall& c, const double* psi, const f
     }
     const unsigned egrid = (unsigned)std::min<long long>(M.E, (long long)sms * 16);
     KTimer kt(&M, VEF_K_RESIDUAL, c.stream);
-    if (P >= kPairMinP && x32) {
-      auto kern = residual_pair_kernel<P, false>;
-      if constexpr (P == 3) {
-        if (form_y) kern = residual_pair_kernel<P, true>;
-      }
-      // one wave of resident CTAs, each walking its elements
-      const size_t smem = S.D * sizeof(float4);
-      int per_sm = 0;
-      VEF_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 128, smem));
-      kern<<<(unsigned)std::min<long long>(M.E, (long long)sms * std::max(1, per_sm)), 128, smem, c.stream>>>(
-          S.D, M.E, M.nx, M.ny, M.nbf, S.omega_dev, c.sigma_t, M.Mmat, M.Gx, M.Gy, M.nds, M.one,
-          M.bvol, c.src_aniso, c.inflow, x32, make_facetab<double>(M.tab), r, norms, S.member_of, recx32, y32,
-          S.members, M.dev_status);
-      VEF_CUDA_TRY(cudaGetLastError());
-      return VEF_OK;
-    }
     auto kern = residual_mf_kernel<P, false>;
     if constexpr (P == 3) {   // the only order whose correction sweeps take y from here
       if (form_y) kern = residual_mf_kernel<P, true>;
@@ -1888,7 +1615,7 @@ static vef_status solve_p(const SweepCall& c, double* psi, vef_info* info) {
   for (int pass = 0; pass < c.max_passes; ++pass) {
     // fixed passes: the last sweep's residual is not formed, and nothing is read back
     if (c.fixed_passes && pass == c.max_passes - 1) break;
-    if ((st = launch_residual<P>(c, psi, pass == 0 ? delta : nullptr, r, norms, y_in_residual)) != VEF_OK) return st;
+    if ((st = launch_residual<P>(c, psi, r, norms, y_in_residual)) != VEF_OK) return st;
     if (!c.fixed_passes) {
       double h[2];
       VEF_CUDA_TRY(cudaMemcpyAsync(h, norms, sizeof(h), cudaMemcpyDeviceToHost, c.stream));
