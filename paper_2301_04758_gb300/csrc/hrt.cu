@@ -14,9 +14,9 @@
 // CTA in shared memory (the map's derivatives and the Eddington tensor evaluated once per
 // Gauss point; D and C1 are the same on every element and come from host tables);
 // hrt_invert_kernel, at a higher occupancy, inverts [[A, G], [D, Ma]] by Gauss-Jordan
-// elimination in registers (diagonal pivots behind a guard, partial pivoting as the fallback),
-// and forms the element's share of the reduced system (the two kernels and the recovery: 2.5 ms
-// at 128^2 Q2, 7.3 before, when divergent lanes and zero components took half of the FP64 issue),
+// elimination with partial pivoting in registers, and forms the element's share of the reduced
+// system (the two kernels and the recovery: 3.0 ms at 128^2 Q2, 7.5 when divergent lanes, zero
+// components and shared-memory traffic took most of the issue),
 //     H_e = C1 W C2,   r_e = C1 (W g + X f),   [[W, X], [Y, Z]] = [[A, G], [D, Ma]]^{-1}.
 // The multiplier system H lambda = r (H = sum_e H_e over the interior faces, not symmetric
 // for a general Eddington tensor) is solved by BiCGStab with a two-level additive Schwarz
@@ -466,16 +466,19 @@ hrt_local_kernel(long long E, int nx, int ny, int qc, const HrtRef<P>* __restric
 }
 
 // Inversion of the assembled local systems and the element's share of the reduced system,
-// apart from the assembly so that it runs many CTAs per SM.  Gauss-Jordan with the matrix in
-// registers (entry idx = i MM + j on thread idx mod T): per step the pivot's row and column
-// are published in shared memory and every entry takes one FMA, a = R_j (-c_i) + a with
-// R = row / pivot, where the pivot's own row and column start from zero (R_k = 1 / pivot,
-// -c_k = 1), so no lane of a warp takes another path.  The diagonal pivots are taken in
-// order: A is positive definite for sigma_t > 0, and so is the Schur complement
-// sigma_a M - D A^{-1} G, with G close to -E : D^T.  A system with a pivot below
-// 2^-kHrtPivotFloor of its row's largest entry, or not finite, is inverted again with partial
-// pivoting (the slow path, from the assembled system).
-constexpr int kHrtPivotFloor = 26;
+// apart from the assembly so that it runs many CTAs per SM.  Gauss-Jordan with partial
+// pivoting and the matrix in registers, rows tr + TR u and columns tc + TC v on thread
+// (tr, tc): per step the pivot's column is already in shared memory, every warp picks the pivot
+// row from it, the row's owners publish R = row / pivot and every entry takes one FMA,
+// a = R_j (-c_i) + a, where the pivot's own row and column start from zero (R_k = 1 / pivot,
+// -c_k = 1), so no lane of a warp takes another path; the owners of the next column publish it
+// as they update it.  The grids of threads leave few idle: 11 x 11 with 3 x 3 entries each for
+// 33 unknowns (p = 2), 28 x 8 with 2 x 7 for 56, 15 x 17 with 6 x 5 for 85.  Rows stay
+// where they are: step k's pivot row perm[k] ends as row k of the inverse, and column j belongs
+// to the right-hand side of equation perm[j].  The pivoting is needed: on optically thin
+// elements A's entries are small against G's, and diagonal pivots left phi an error of 2e-10 to
+// 4e-9 at sigma_t = 1e-7 (1e-16 with pivoting; one element, p = 1..4).  It costs 0.5 of the
+// 3.0 ms at 128^2 Q2, 1.9 of 32.5 at Q4.
 template <int P>
 struct HrtInvSmem {
   using S = HrtShape<P>;
@@ -484,16 +487,15 @@ struct HrtInvSmem {
   double gf[S::MM];                  // g, f
   double T1[S::NL4][S::NL4];         // rows of W C2 at the face unknowns
   double u[S::NL4];                  // W g + X f there
-  double row[S::MM], col[S::MM];     // the pivot's row and column, as published
-  double R[S::MM], nc[S::MM];        // row / pivot and -column
-  double colk[S::MM];
-  double inv;                        // reciprocal of the current pivot (slow path)
-  int scale[S::MM];                  // high word of each row's largest magnitude
-  int perm[S::MM];
-  int piv;
+  double col[2][S::MM];              // the pivot's column, this step's and the next one's
+  double R[S::MM];                   // row / pivot
+  int perm[S::MM], step[S::MM];      // pivot row of each step, and its inverse
 };
 template <int P> struct HrtInvShape {
-  static constexpr int T = P <= 2 ? 128 : 256, NR = (HrtShape<P>::MM * HrtShape<P>::MM + T - 1) / T;
+  static constexpr int MM = HrtShape<P>::MM;
+  static constexpr int TR = P == 1 ? 8 : P == 2 ? 11 : P == 3 ? 28 : 15, TC = P == 1 ? 16 : P == 2 ? 11 : P == 3 ? 8 : 17;
+  static constexpr int NU = (MM + TR - 1) / TR, NV = (MM + TC - 1) / TC, T = (TR * TC + 31) / 32 * 32;
+  static_assert(NV * TC == MM, "whole columns");
 };
 
 template <int P>
@@ -501,124 +503,108 @@ __global__ void __launch_bounds__(HrtInvShape<P>::T)
 hrt_invert_kernel(long long E, int nx, int ny, const HrtRef<P>* __restrict__ ref, HrtOut out, unsigned int* status) {
   using S = HrtShape<P>;
   constexpr int N = S::N, NJ = S::NJ, MM = S::MM, LD = S::LD, NL = S::NL, NL4 = S::NL4, NX = S::NX;
-  constexpr int T = HrtInvShape<P>::T, NR = HrtInvShape<P>::NR;
+  using I = HrtInvShape<P>;
+  constexpr int T = I::T, TR = I::TR, TC = I::TC, NU = I::NU, NV = I::NV, RPW = (MM + 31) / 32;
+  constexpr unsigned FULL = 0xffffffffu;
   extern __shared__ __align__(16) unsigned char hrt_inv_smem[];
   HrtInvSmem<P>& sm = *reinterpret_cast<HrtInvSmem<P>*>(hrt_inv_smem);
-  const int tid = threadIdx.x, nth = T;
+  const int tid = threadIdx.x, lane = tid & 31, nth = T;
+  // this thread's rows and columns (a thread past the grid holds row MM and up: none)
+  const int tr = tid < TR * TC ? tid / TC : MM, tc = tid < TR * TC ? tid % TC : 0;
   // the RT unknown with a normal flux on face f at tangential node b (C1's columns)
   auto face_unknown = [](int f, int b) {
     return f == 3 ? (P + 2) * b : f == 1 ? P + 1 + (P + 2) * b : f == 0 ? NX + b : NX + b + (P + 1) * (P + 1);
   };
   for (long long e = blockIdx.x; e < E; e += gridDim.x) {
     __syncthreads();
-    for (int i = tid; i < MM; i += nth) sm.scale[i] = 0;
     for (int idx = tid; idx < NL4 * NJ; idx += nth) (&sm.C2[0][0])[idx] = out.C2[(size_t)e * NJ * NL4 + idx];
     for (int a = tid; a < MM; a += nth) sm.gf[a] = a < NJ ? out.g[(size_t)e * NJ + a] : out.f[(size_t)e * N + a - NJ];
     double* Lg = out.Li + (size_t)e * MM * MM;
-    double a[NR];
+    double a[NU][NV];
+#pragma unroll
+    for (int u = 0; u < NU; ++u) {
+      const int i = tr + TR * u;
+#pragma unroll
+      for (int v = 0; v < NV; ++v) a[u][v] = i < MM ? Lg[i * MM + tc + TC * v] : 0.0;
+      if (i < MM && tc == 0) sm.col[0][i] = a[u][0];
+    }
+    unsigned used = 0;   // which of rows lane, lane + 32, ... have been pivots
+    for (int k = 0; k < MM; ++k) {
+      __syncthreads();
+      const double* col = sm.col[k & 1];
+      // the largest magnitude of the rows left (not a NaN; the lowest such row): high words,
+      // then low words, then the index; -1 where a row takes no part
+      int hi[RPW], best = -1;
+#pragma unroll
+      for (int q = 0; q < RPW; ++q) {
+        const int i = lane + 32 * q;
+        hi[q] = i < MM && !((used >> q) & 1) ? __double2hiint(col[i]) & 0x7fffffff : -1;
+        if (hi[q] > 0x7ff00000) hi[q] = -2;
+        best = max(best, hi[q]);
+      }
+      best = __reduce_max_sync(FULL, best);
+      unsigned lo[RPW], blo = 0;
+#pragma unroll
+      for (int q = 0; q < RPW; ++q) {
+        const int i = lane + 32 * q;
+        lo[q] = i < MM ? (unsigned)__double2loint(col[i]) : 0;
+        if (hi[q] == best) blo = max(blo, lo[q]);
+      }
+      blo = __reduce_max_sync(FULL, blo);
+      int pr = MM;
+#pragma unroll
+      for (int q = RPW - 1; q >= 0; --q) {
+        if (best >= 0 ? hi[q] == best && lo[q] == blo : hi[q] == -2) pr = lane + 32 * q;
+      }
+      pr = __reduce_min_sync(FULL, pr);
+      if ((pr & 31) == lane) used |= 1u << (pr >> 5);
+      const double piv = col[pr];
+      if (tid == 0) {
+        sm.perm[k] = pr;
+        sm.step[pr] = k;
+        if (best < 0 || !(fabs(piv) > 1e-300)) atomicOr(status, kDevSingular);
+      }
+      const int ur = pr / TR, vk = k / TC, vn = (k + 1) / TC;
+      const bool own_row = tr == pr - ur * TR, own_col = tc == k - vk * TC, own_next = tc == k + 1 - vn * TC;
+      if (own_row) {
+        const double inv = 1.0 / piv;
+#pragma unroll
+        for (int v = 0; v < NV; ++v) {
+          double x = a[0][v];
+#pragma unroll
+          for (int u = 1; u < NU; ++u) x = u == ur ? a[u][v] : x;
+          sm.R[tc + TC * v] = own_col && v == vk ? inv : x * inv;
+        }
+      }
+      __syncthreads();
+      double R[NV];
+#pragma unroll
+      for (int v = 0; v < NV; ++v) R[v] = sm.R[tc + TC * v];
+#pragma unroll
+      for (int u = 0; u < NU; ++u) {
+        const int i = tr + TR * u;
+        const bool prow = own_row && u == ur;
+        const double c = i < MM ? (prow ? 1.0 : -col[i]) : 0.0;
+        double next = 0.0;
+#pragma unroll
+        for (int v = 0; v < NV; ++v) {
+          a[u][v] = fma(c, R[v], prow || (own_col && v == vk) ? 0.0 : a[u][v]);
+          next = v == vn ? a[u][v] : next;
+        }
+        if (own_next && i < MM) sm.col[(k + 1) & 1][i] = next;
+      }
+    }
     __syncthreads();
 #pragma unroll
-    for (int r = 0; r < NR; ++r) {
-      const int idx = tid + r * T, i = idx / MM;
-      a[r] = idx < MM * MM ? Lg[idx] : 0.0;
-      if (idx < MM * MM) atomicMax(&sm.scale[i], __double2hiint(a[r]) & 0x7fffffff);
-    }
-    bool bad = false;
-    for (int k = 0; k < MM; ++k) {
+    for (int u = 0; u < NU; ++u) {
+      const int i = tr + TR * u;
+      if (i < MM) {
 #pragma unroll
-      for (int r = 0; r < NR; ++r) {
-        const int idx = tid + r * T, i = idx / MM, j = idx - i * MM;
-        if (i == k) sm.row[j] = a[r];
-        if (j == k && i < MM) sm.col[i] = a[r];
-      }
-      __syncthreads();
-      if (tid < (MM + 31) / 32 * 32) {
-        const double piv = sm.row[k];
-        const int mag = __double2hiint(piv) & 0x7fffffff;
-        bad = bad || mag < sm.scale[k] - (kHrtPivotFloor << 20) || mag >= (2000 << 20) || mag < (50 << 20);
-        const double inv = pivot_rcp(piv);
-        if (tid < MM) {
-          sm.R[tid] = tid == k ? inv : sm.row[tid] * inv;
-          sm.nc[tid] = tid == k ? 1.0 : -sm.col[tid];
-        }
-      }
-      __syncthreads();
-#pragma unroll
-      for (int r = 0; r < NR; ++r) {
-        const int idx = tid + r * T, i = idx / MM, j = idx - i * MM;
-        const double old = i == k || j == k ? 0.0 : a[r];
-        if (idx < MM * MM) a[r] = fma(sm.nc[i], sm.R[j], old);
+        for (int v = 0; v < NV; ++v) sm.L[sm.step[i] * LD + sm.perm[tc + TC * v]] = a[u][v];
       }
     }
-    if (!__syncthreads_or(bad)) {
-#pragma unroll
-      for (int r = 0; r < NR; ++r) {
-        const int idx = tid + r * T;
-        if (idx < MM * MM) {
-          sm.L[(idx / MM) * LD + idx % MM] = a[r];
-          Lg[idx] = a[r];
-        }
-      }
-      __syncthreads();
-    } else {
-      for (int idx = tid; idx < MM * MM; idx += nth) sm.L[(idx / MM) * LD + idx % MM] = Lg[idx];
-      __syncthreads();
-      for (int k = 0; k < MM; ++k) {
-        if (tid < 32) {
-          double best = -1.0;
-          int bi = k;
-          for (int i = k + tid; i < MM; i += 32) {
-            const double v = fabs(sm.L[i * LD + k]);
-            if (v > best) { best = v; bi = i; }
-          }
-          for (int off = 16; off > 0; off >>= 1) {
-            const double ob = __shfl_xor_sync(0xffffffffu, best, off);
-            const int oi = __shfl_xor_sync(0xffffffffu, bi, off);
-            if (ob > best || (ob == best && oi < bi)) { best = ob; bi = oi; }
-          }
-          if (tid == 0) {
-            sm.piv = bi;
-            sm.perm[k] = bi;
-            sm.inv = 1.0 / sm.L[bi * LD + k];   // one FP64 division per step, not one per thread
-            if (!(best > 1e-300)) atomicOr(status, kDevSingular);
-          }
-        }
-        __syncthreads();
-        const int pr = sm.piv;
-        if (pr != k)
-          for (int j = tid; j < MM; j += nth) {
-            const double tmp = sm.L[k * LD + j];
-            sm.L[k * LD + j] = sm.L[pr * LD + j];
-            sm.L[pr * LD + j] = tmp;
-          }
-        __syncthreads();
-        const double inv = sm.inv;
-        for (int i = tid; i < MM; i += nth) sm.colk[i] = sm.L[i * LD + k];
-        __syncthreads();
-        for (int j = tid; j < MM; j += nth)
-          if (j != k) sm.L[k * LD + j] *= inv;
-        __syncthreads();
-        for (int idx = tid; idx < MM * MM; idx += nth) {
-          const int i = idx / MM, j = idx % MM;
-          if (i == k) continue;
-          if (j == k) sm.L[i * LD + k] = -sm.colk[i] * inv;
-          else sm.L[i * LD + j] -= sm.colk[i] * sm.L[k * LD + j];
-        }
-        if (tid == 0) sm.L[k * LD + k] = inv;
-        __syncthreads();
-      }
-      for (int k = MM - 1; k >= 0; --k) {   // undo the row interchanges as column interchanges
-        const int pr = sm.perm[k];
-        if (pr != k)
-          for (int i = tid; i < MM; i += nth) {
-            const double tmp = sm.L[i * LD + k];
-            sm.L[i * LD + k] = sm.L[i * LD + pr];
-            sm.L[i * LD + pr] = tmp;
-          }
-        __syncthreads();
-      }
-      for (int idx = tid; idx < MM * MM; idx += nth) Lg[idx] = sm.L[(idx / MM) * LD + idx % MM];
-    }
+    __syncthreads();
+    for (int idx = tid; idx < MM * MM; idx += nth) Lg[idx] = sm.L[(idx / MM) * LD + idx % MM];
     // W C2 and W g + X f at the unknowns with a normal flux on a face (the others have zero
     // columns in C1), then H_e = C1 (W C2) and r_e = C1 (W g + X f)
     for (int idx = tid; idx < NL4 * NL4 + NL4; idx += nth) {

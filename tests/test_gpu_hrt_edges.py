@@ -1,0 +1,46 @@
+"""Edges of the hybridized VEF solve: thin elements whose inversion needs pivoting, dot products
+near the end of FP64's range, status bits after a solve that fails, bounded grid barriers, and
+meshes whose Krylov tiles are cut, empty or several to a CTA."""
+import time
+
+import numpy as np
+import pytest
+
+from _gpu import dev, host, rel, random_problem
+from _hrt_exact import exact_problem
+from oracle.hrt import HRT
+from oracle.transport import Discretization, sweep as o_sweep
+
+pytestmark = pytest.mark.gpu
+
+
+def _solve(mesh, v, **kw):
+    phi, J, lam, info = mesh.hrt_solve(dev(v["sigma_t"]), dev(v["sigma_s"]), dev(v["phi_tr"]), dev(v["P_tr"]),
+                                       dev(v["Eb"]), dev(v["Jin"]), dev(v["Q0"]), dev(v["Q1"]), **kw)
+    return host(phi), host(J), host(lam), info
+
+
+@pytest.mark.parametrize("p", [1, 2, 3, 4])
+@pytest.mark.parametrize("sigma_t", [1e-7, 1e-3])
+def test_thin_element_keeps_the_digits_of_phi(lib, p, sigma_t):
+    """One optically thin element: A's pivots are small against G's entries and an elimination
+    that takes them all the same loses log10(1 / sigma_t) digits of phi.  Relative changes of
+    2^-52 in the entries of the local system move phi by less than 2^-51, so with at most 85
+    elimination steps of a few roundings each phi agrees to 85 x 8 x 2^-53 < 1e-13 with the
+    system's solution in 50 digits."""
+    import mpmath as mp
+    from paper_2301_04758_gb300.api import Mesh
+    disc = Discretization(1, 1, 3, 0.05, p)
+    h, nq = HRT(disc), disc.nq
+    one = np.ones((1, disc.n))
+    v = dict(sigma_t=np.full(1, sigma_t), sigma_s=np.full(1, 0.9 * sigma_t), phi_tr=one,
+             P_tr=np.stack([one / 3, 0 * one, one / 3]), Eb=np.full((4, nq), 0.5), Jin=np.full((4, nq), -0.1),
+             Q0=one, Q1=np.zeros((2, 1, disc.n)))
+    Eq, Ef = h.eddington_data(v["phi_tr"], v["P_tr"])
+    L, _, _, g, f = h.element(0, v["sigma_t"], v["sigma_t"] - v["sigma_s"], Eq, Ef, v["Eb"], v["Jin"],
+                              np.ones((1, nq * nq)))
+    with mp.workdps(50):
+        x = mp.lu_solve(mp.matrix(L.tolist()), mp.matrix(np.concatenate([g, f]).tolist()))
+    ref = np.array([float(t) for t in x])[h.nJ:]
+    phi = _solve(Mesh(1, 1, 3, p, 0.05), v)[0]
+    assert rel(phi[0], ref) < 1e-13
