@@ -215,6 +215,7 @@ Schedule* get_schedule(Mesh* mesh, const double* omega, const double* weights, i
                        cudaStream_t stream, vef_status* st);
 // Waits for `stream`, reads and clears the handle's device status word, maps it to a status.
 vef_status collect_status(Mesh& M, cudaStream_t stream, vef_info* info);
+vef_status collect_status_failed(Mesh& M, cudaStream_t stream, vef_status st);
 
 }  // namespace vef
 

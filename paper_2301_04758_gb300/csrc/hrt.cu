@@ -1752,7 +1752,7 @@ static inline unsigned nblk(long long n, int bs) { return (unsigned)((n + bs - 1
 
 template <int P>
 static vef_status hrt_run(Mesh& M, const HrtIn& in, double tol, int max_iter, double* phi, double* J,
-                          double* lambda, vef_hrt_info* info, cudaStream_t s) {
+                          double* lambda, vef_hrt_info* info, cudaStream_t s, bool& launched) {
   using S = HrtShape<P>;
   const long long E = M.E;
   const long long nfaces = (long long)(M.nx - 1) * M.ny + (long long)M.nx * (M.ny - 1);
@@ -1836,6 +1836,7 @@ static vef_status hrt_run(Mesh& M, const HrtIn& in, double tol, int max_iter, do
   VEF_CUDA_TRY(cudaGetDevice(&dev));
   VEF_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   VEF_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&inv_per_sm, hrt_invert_kernel<P>, HrtInvShape<P>::T, ismem));
+  launched = true;
   {
     KTimer kt(&M, VEF_K_HRT, s);
     hrt_local_kernel<P><<<(unsigned)std::min<long long>(E, (long long)sms * 8), 256, smem, s>>>(
@@ -1934,12 +1935,13 @@ extern "C" vef_status vef_hrt_solve(vef_mesh mesh, const double* sigma_t, const 
   HrtIn in{M.ctrl_dev, M.Mmat, M.nds, sigma_t, sigma_s, phi_tr, P_tr, Eb, Jin, Q0, Q1};
   cudaStream_t s = (cudaStream_t)stream;
   vef_status st;
+  bool launched = false;
   switch (M.p) {
-    case 1: st = hrt_run<1>(M, in, tol, max_iter, phi, J, lambda, info, s); break;
-    case 2: st = hrt_run<2>(M, in, tol, max_iter, phi, J, lambda, info, s); break;
-    case 3: st = hrt_run<3>(M, in, tol, max_iter, phi, J, lambda, info, s); break;
-    default: st = hrt_run<4>(M, in, tol, max_iter, phi, J, lambda, info, s); break;
+    case 1: st = hrt_run<1>(M, in, tol, max_iter, phi, J, lambda, info, s, launched); break;
+    case 2: st = hrt_run<2>(M, in, tol, max_iter, phi, J, lambda, info, s, launched); break;
+    case 3: st = hrt_run<3>(M, in, tol, max_iter, phi, J, lambda, info, s, launched); break;
+    default: st = hrt_run<4>(M, in, tol, max_iter, phi, J, lambda, info, s, launched); break;
   }
-  if (st != VEF_OK) return st;
-  return collect_status(M, s, nullptr);
+  if (st == VEF_OK) return collect_status(M, s, nullptr);
+  return launched ? collect_status_failed(M, s, st) : st;
 }

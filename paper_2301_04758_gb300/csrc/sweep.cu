@@ -1690,14 +1690,21 @@ static vef_status launch_bvol(Mesh& M, const double* sigma_s, const double* phi_
   return VEF_OK;
 }
 
-// Read back and clear the device status; map to a vef_status.
-vef_status collect_status(Mesh& M, cudaStream_t stream, vef_info* info) {
-  unsigned int h[8];
-  VEF_CUDA_TRY(cudaMemcpyAsync(h, M.dev_status, sizeof(h), cudaMemcpyDeviceToHost, stream));
+// Read the device status word and its counters back into h[8] and clear them.
+static vef_status drain_status(Mesh& M, cudaStream_t stream, unsigned int* h) {
+  VEF_CUDA_TRY(cudaMemcpyAsync(h, M.dev_status, 8 * sizeof(unsigned int), cudaMemcpyDeviceToHost, stream));
   VEF_CUDA_TRY(cudaStreamSynchronize(stream));
   unsigned int zero[8] = {0, 0, 0, 0, 0, 0, 0, 0};
   VEF_CUDA_TRY(cudaMemcpyAsync(M.dev_status, zero, sizeof(zero), cudaMemcpyHostToDevice, stream));
   VEF_CUDA_TRY(cudaStreamSynchronize(stream));
+  return VEF_OK;
+}
+
+// Read back and clear the device status; map to a vef_status.
+vef_status collect_status(Mesh& M, cudaStream_t stream, vef_info* info) {
+  unsigned int h[8];
+  const vef_status st = drain_status(M, stream, h);
+  if (st != VEF_OK) return st;
   const unsigned bits = h[0] | h[4];
   if (info) {
     info->timed_out = (bits & kDevTimeout) ? 1 : 0;
@@ -1705,11 +1712,25 @@ vef_status collect_status(Mesh& M, cudaStream_t stream, vef_info* info) {
     info->pivoted_tasks = (long long)h[kStatusPivoted];
   }
   if (bits & kDevBounds) { set_last_error("bounds check: a kernel met an index outside its array"); return VEF_ERR_BOUNDS; }
-  if (bits & kDevTimeout) { set_last_error("a sweep dependency wait ran out"); return VEF_ERR_TIMEOUT; }
+  if (bits & kDevTimeout) { set_last_error("a bounded device-side wait ran out"); return VEF_ERR_TIMEOUT; }
   if (bits & kDevSingular) { set_last_error("singular local element system"); return VEF_ERR_NOT_CONVERGED; }
   if (bits & kDevNotConverged) { set_last_error("an iteration reached its cap"); return VEF_ERR_NOT_CONVERGED; }
   if (bits & kDevNonpositive) { set_last_error("non-positive closure denominator"); return VEF_ERR_NONPOSITIVE_DENOM; }
   return VEF_OK;
+}
+
+// The same for a call that has failed with st: the status is cleared, so that it does not reach
+// the next call, and st stands, unless st is a missing convergence and a kernel recorded why its
+// result is worthless (a wait that ran out, an index out of range).
+vef_status collect_status_failed(Mesh& M, cudaStream_t stream, vef_status st) {
+  unsigned int h[8];
+  const vef_status cs = drain_status(M, stream, h);
+  if (st != VEF_ERR_NOT_CONVERGED) return st;
+  if (cs != VEF_OK) return cs;
+  const unsigned bits = h[0] | h[4];
+  if (bits & kDevBounds) { set_last_error("bounds check: a kernel met an index outside its array"); return VEF_ERR_BOUNDS; }
+  if (bits & kDevTimeout) { set_last_error("a bounded device-side wait ran out"); return VEF_ERR_TIMEOUT; }
+  return st;
 }
 
 static vef_status check_common(vef_mesh mesh, const double* omega, const double* weights, int D,

@@ -44,3 +44,33 @@ def test_thin_element_keeps_the_digits_of_phi(lib, p, sigma_t):
     ref = np.array([float(t) for t in x])[h.nJ:]
     phi = _solve(Mesh(1, 1, 3, p, 0.05), v)[0]
     assert rel(phi[0], ref) < 1e-13
+
+
+@pytest.mark.parametrize("kind", ["nan_moment", "pending_timeout"])
+def test_a_failed_solve_leaves_no_status_behind(lib, kind):
+    """A solve that ends without converging reports what its kernels recorded (a wait that ran
+    out before the missing convergence) and leaves the mesh clean: the next sweep and the next
+    solve succeed."""
+    from paper_2301_04758_gb300 import _lib
+    from paper_2301_04758_gb300.api import Mesh
+    nx, ny, p = 6, 5, 2
+    v = exact_problem(nx, ny, p, 830)
+    prob = random_problem(nx, ny, 1, 0.0, p, 4, seed=831)
+    mesh = Mesh(nx, ny, 1, p, 0.0)
+    bad, kw, want = dict(v), dict(tol=1e-13), _lib.VEF_ERR_NOT_CONVERGED
+    if kind == "nan_moment":
+        bad["phi_tr"] = v["phi_tr"].copy()
+        bad["phi_tr"][7, 0] = np.nan
+    else:
+        kw, want = dict(tol=1e-13, max_iter=1), _lib.VEF_ERR_TIMEOUT
+        assert lib.vef_mesh_inject_status(mesh.handle, _lib.VEF_STATUS_TIMEOUT, None) == _lib.VEF_OK
+    with pytest.raises(_lib.VefError) as err:
+        _solve(mesh, bad, **kw)
+    assert err.value.status == want, err.value
+    psi, info = mesh.sweep(dev(prob["sigma_t"]), dev(prob["sigma_s"]), prob["omega"], prob["weights"],
+                           phi_in=dev(prob["phi_in"]), source=dev(prob["source"]), inflow=dev(prob["inflow"]), info=True)
+    ref = o_sweep(Discretization(nx, ny, 1, 0.0, p), prob["omega"], prob["weights"], prob["sigma_t"], prob["sigma_s"],
+                  phi_in=prob["phi_in"], source=prob["source"], inflow=prob["inflow"])
+    assert rel(host(psi), ref) < 1e-12 and info["timed_out"] == 0
+    phi, J, lam, _ = _solve(mesh, v, tol=1e-13)
+    assert rel(phi, v["phi"]) < 1e-10 and rel(J, v["J"]) < 1e-10 and rel(lam, v["lam"]) < 1e-10
