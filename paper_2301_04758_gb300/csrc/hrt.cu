@@ -1254,11 +1254,12 @@ struct KryScal {
 };
 
 // a / b to within two ulp: the approximate reciprocal refined by two Newton-Raphson steps
-// (pivot_rcp), at a third of a division's dependent FP64 operations; an operand outside the
-// reciprocal's range divides
+// (pivot_rcp), at a third of a division's dependent FP64 operations; a b of magnitude 2^1021 and
+// up, whose reciprocal is below the normal range and would come out as zero, and results that
+// are not finite divide
 __device__ __forceinline__ double kry_quot(double a, double b) {
   const double q = a * pivot_rcp(b);
-  return isfinite(q) ? q : a / b;
+  return isfinite(q) && (__double2hiint(b) & 0x7fffffff) < ((1021 + 1023) << 20) ? q : a / b;
 }
 
 // the sums over the tiles of nq <= 4 dots q, warp w summing dot q[w] in a fixed order, into

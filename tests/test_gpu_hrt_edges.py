@@ -74,3 +74,21 @@ def test_a_failed_solve_leaves_no_status_behind(lib, kind):
     assert rel(host(psi), ref) < 1e-12 and info["timed_out"] == 0
     phi, J, lam, _ = _solve(mesh, v, tol=1e-13)
     assert rel(phi, v["phi"]) < 1e-10 and rel(J, v["J"]) < 1e-10 and rel(lam, v["lam"]) < 1e-10
+
+
+def test_dot_products_near_the_end_of_the_range(lib):
+    """Sources scaled until ||r||^2 = 2^1021.7: the first iteration divides by r_hat . v between
+    2^1022 and 2^1024, whose reciprocal is below FP64's normal range.  The problem is linear, so
+    the solution scales with the sources."""
+    from paper_2301_04758_gb300.api import Mesh
+    p = 2
+    v = exact_problem(2, 1, p, 840)
+    disc = Discretization(2, 1, 1, 0.0, p)
+    h = HRT(disc)
+    ref = h.solve(v["sigma_t"], v["sigma_s"], *h.eddington_data(v["phi_tr"], v["P_tr"]), v["Eb"], v["Jin"],
+                  np.einsum("qj,ej->eq", disc.B, v["Q0"]), np.einsum("qj,cej->eqc", disc.B, v["Q1"]))
+    scale = 2.0 ** 510.85 / np.linalg.norm(ref["r"])
+    big = dict(v, Jin=scale * v["Jin"], Q0=scale * v["Q0"], Q1=scale * v["Q1"])
+    phi, J, lam, info = _solve(Mesh(2, 1, 1, p, 0.0), big, tol=1e-13)
+    for got, key in ((phi, "phi"), (J, "J"), (lam, "lam")):
+        assert rel(got / scale, v[key]) < 1e-11, info
