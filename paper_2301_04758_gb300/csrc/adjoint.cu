@@ -725,7 +725,7 @@ static vef_status launch_adjoint_cta(Mesh& M, Schedule& S, AdjArgs a, cudaStream
                                                           (double*)M.ybuf);
     VEF_CUDA_TRY(cudaGetLastError());
   }
-  VEF_CUDA_TRY(cudaFuncSetAttribute(adjoint_cta_kernel<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  if ((st = allow_dynamic_smem<adjoint_cta_kernel<P>>()) != VEF_OK) return st;
   KTimer kt(&M, VEF_K_ADJOINT, s);   // the backward sweep and the gradient post-pass
   adjoint_cta_kernel<P><<<(unsigned)S.D, Sh::kThreads, smem, s>>>(a);
   VEF_CUDA_TRY(cudaGetLastError());

@@ -4,6 +4,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "common.h"
 
 namespace vef {
@@ -199,6 +201,26 @@ __device__ __forceinline__ void cluster_wait() {
 
 template <typename T>
 __device__ __forceinline__ T ldcg(const T* p) { return __ldcg(p); }
+
+// Allows Kernel all the dynamic shared memory a CTA can have beside its static one.  The limit is
+// the function's, for every thread of the process: set to what one call needs, it would refuse
+// the launch of a larger call made from another thread in between.
+template <auto Kernel>
+inline vef_status allow_dynamic_smem() {
+  static std::atomic<int> room{-1};
+  int r = room.load(std::memory_order_relaxed);
+  if (r < 0) {
+    cudaFuncAttributes fa;
+    int dev = 0, optin = 0;
+    VEF_CUDA_TRY(cudaFuncGetAttributes(&fa, Kernel));
+    VEF_CUDA_TRY(cudaGetDevice(&dev));
+    VEF_CUDA_TRY(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+    r = optin - (int)fa.sharedSizeBytes;
+    room.store(r, std::memory_order_relaxed);
+  }
+  VEF_CUDA_TRY(cudaFuncSetAttribute(Kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, r));
+  return VEF_OK;
+}
 
 // Table of 1D Lagrange values for kernels templated on the real type.
 template <typename T>

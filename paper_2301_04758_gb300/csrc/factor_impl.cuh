@@ -1312,8 +1312,7 @@ static vef_status launch_group_factor(Schedule& S, const void* rec, cudaStream_t
   if ((st = warp_launch(group_factor_warp_kernel<P, T, 32>, lo[2], up[2])) != VEF_OK) return st;
   if (S.ngroups > up[2]) {
     const size_t smem = (size_t)S.max_nt * S.max_nt * sizeof(double);
-    VEF_CUDA_TRY(cudaFuncSetAttribute(group_factor_kernel<P, T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)smem));
+    if ((st = allow_dynamic_smem<group_factor_kernel<P, T>>()) != VEF_OK) return st;
     group_factor_kernel<P, T><<<(unsigned)(S.ngroups - up[2]), kGroupThreads, smem, stream>>>(
         (int)up[2], S.grp_slot, S.grp_nt, S.grp_toff, S.slot_first, S.slot_count, S.member_nbpos,
         (const T*)rec, S.members, (T*)*gp, status);

@@ -1829,10 +1829,10 @@ static vef_status hrt_run(Mesh& M, const HrtIn& in, double tol, int max_iter, do
   k.st = reinterpret_cast<KState*>(take(sizeof(KState) / sizeof(double)));
   HrtOut out{Li, C2, g, f, He, re};
   const size_t smem = sizeof(HrtSmem<P>), ismem = sizeof(HrtInvSmem<P>);
-  VEF_CUDA_TRY(cudaFuncSetAttribute(hrt_local_kernel<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  VEF_CUDA_TRY(cudaFuncSetAttribute(hrt_invert_kernel<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ismem));
   const size_t csmem = (size_t)nc * (nc | 1) * sizeof(float);
-  VEF_CUDA_TRY(cudaFuncSetAttribute(hrt_coarse_pivot_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)csmem));
+  if ((st = allow_dynamic_smem<hrt_local_kernel<P>>()) != VEF_OK) return st;
+  if ((st = allow_dynamic_smem<hrt_invert_kernel<P>>()) != VEF_OK) return st;
+  if ((st = allow_dynamic_smem<hrt_coarse_pivot_kernel>()) != VEF_OK) return st;
   int dev = 0, sms = 0, inv_per_sm = 0;
   VEF_CUDA_TRY(cudaGetDevice(&dev));
   VEF_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
@@ -1861,7 +1861,7 @@ static vef_status hrt_run(Mesh& M, const HrtIn& in, double tol, int max_iter, do
     hs.tol2 = tol * tol;
     VEF_CUDA_TRY(cudaMemcpyAsync(k.st, &hs, sizeof(KState), cudaMemcpyHostToDevice, s));
     const size_t ksmem = tile_smem();
-    VEF_CUDA_TRY(cudaFuncSetAttribute(kry_solve_kernel<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ksmem));
+    if ((st = allow_dynamic_smem<kry_solve_kernel<P>>()) != VEF_OK) return st;
     int per_sm = 0;
     VEF_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kry_solve_kernel<P>, kKT, ksmem));
     int grid = std::max(1, std::min(k.ntiles, sms * std::max(1, per_sm)));

@@ -1382,8 +1382,8 @@ static vef_status launch_apply(const SweepCall& c, const SweepArgs<T>& a) {
 }
 
 // cluster launch configuration of the sweep kernels (clusters x cs CTAs of warps x 32)
-template <int P, typename T, typename K>
-static vef_status cluster_config(K kernel, long long clusters, int cs, int warps, cudaStream_t stream,
+template <int P, typename T, auto Kernel>
+static vef_status cluster_config(long long clusters, int cs, int warps, cudaStream_t stream,
                                  cudaLaunchConfig_t& cfg, cudaLaunchAttribute* attr) {
   cfg = cudaLaunchConfig_t{};
   cfg.gridDim = dim3((unsigned)(clusters * cs));
@@ -1396,9 +1396,9 @@ static vef_status cluster_config(K kernel, long long clusters, int cs, int warps
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   cfg.dynamicSmemBytes = sweep_smem_bytes<P, T>(warps, cs * warps);
-  VEF_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)cfg.dynamicSmemBytes));
-  if (cs > 8) VEF_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+  const vef_status st = allow_dynamic_smem<Kernel>();
+  if (st != VEF_OK) return st;
+  if (cs > 8) VEF_CUDA_TRY(cudaFuncSetAttribute(Kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
   return VEF_OK;
 }
 
@@ -1421,7 +1421,7 @@ static vef_status auto_tile(int D, int& cs_out, int& warps_out) {
   for (int cs = 8; cs >= 1; --cs) {
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr[1];
-    vef_status st = cluster_config<P, T>(sweep_kernel<P, T, MODE>, 1, cs, warps_out, nullptr, cfg, attr);
+    vef_status st = cluster_config<P, T, sweep_kernel<P, T, MODE>>(1, cs, warps_out, nullptr, cfg, attr);
     if (st != VEF_OK) return st;
     int fit = 0;
     VEF_CUDA_TRY(cudaOccupancyMaxActiveClusters(&fit, sweep_kernel<P, T, MODE>, &cfg));
@@ -1449,7 +1449,8 @@ static vef_status launch_sweep_cta(const SweepCall& c, SweepArgs<T>& a) {
   a.tr_bytes = tr;
   const size_t smem = (size_t)Sh::kGroup + Sh::kBars + tr + (size_t)rounds * Sh::kRound;
   auto kern = sweep_cta_kernel<P, T, MODE>;
-  VEF_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  vef_status st = allow_dynamic_smem<sweep_cta_kernel<P, T, MODE>>();
+  if (st != VEF_OK) return st;
   // the SMs the directions leave free apply A^{-1} inside the same (cooperative) launch
   int dev = 0, sms = 0, per_sm = 0;
   VEF_CUDA_TRY(cudaGetDevice(&dev));
@@ -1477,7 +1478,7 @@ static vef_status launch_sweep_cta(const SweepCall& c, SweepArgs<T>& a) {
   a.nd = S.D;
   a.nmem = S.members;
   const size_t flag_bytes = (size_t)S.D * a.bands * sizeof(int);
-  vef_status st = ensure_buffer((void**)&M.ready_flags, &M.ready_cap, flag_bytes);
+  st = ensure_buffer((void**)&M.ready_flags, &M.ready_cap, flag_bytes);
   if (st != VEF_OK) return st;
   a.ready = M.ready_flags;
   VEF_CUDA_TRY(cudaMemsetAsync(M.ready_flags, 0, flag_bytes, c.stream));
@@ -1530,8 +1531,8 @@ static vef_status launch_sweep(const SweepCall& c0, const double* rhs, T* out) {
   if (!c.y_ready && (st = launch_apply<P, T, MODE>(c, a)) != VEF_OK) return st;
   cudaLaunchConfig_t cfg;
   cudaLaunchAttribute attr[1];
-  if ((st = cluster_config<P, T>(sweep_kernel<P, T, MODE>, c.S->D, c.cluster_size, c.cta_warps, c.stream,
-                                 cfg, attr)) != VEF_OK)
+  if ((st = cluster_config<P, T, sweep_kernel<P, T, MODE>>(c.S->D, c.cluster_size, c.cta_warps, c.stream, cfg,
+                                                          attr)) != VEF_OK)
     return st;
   KTimer kt(c.mesh, VEF_K_SWEEP, c.stream);
   VEF_CUDA_TRY(cudaLaunchKernelEx(&cfg, sweep_kernel<P, T, MODE>, a));
@@ -1948,7 +1949,8 @@ static vef_status batch_launch_class(vef_batch_s& B, BatchClass& C, int tile, cu
   if (tile == kBatchCta) {
     using Sh = CtaShape<P, double>;
     auto kern = sweep_cta_batch_kernel<P, double, 0>;
-    VEF_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C.cta_smem));
+    const vef_status st = allow_dynamic_smem<sweep_cta_batch_kernel<P, double, 0>>();
+    if (st != VEF_OK) return st;
     KTimer kt(B.meshes[C.probs[0]], VEF_K_SWEEP, s);
     kern<<<(unsigned)C.clusters, Sh::kThreads, C.cta_smem, s>>>((const SweepArgs<double>*)C.tab_dev,
                                                                (const int2*)C.cmap);
@@ -1958,7 +1960,7 @@ static vef_status batch_launch_class(vef_batch_s& B, BatchClass& C, int tile, cu
   const int cs = std::min(16, std::max(1, tile / 100)), warps = std::min(16, std::max(1, tile % 100));
   cudaLaunchConfig_t cfg;
   cudaLaunchAttribute attr[1];
-  vef_status st = cluster_config<P, double>(sweep_batch_kernel<P, double, 0>, C.clusters, cs, warps, s, cfg, attr);
+  vef_status st = cluster_config<P, double, sweep_batch_kernel<P, double, 0>>(C.clusters, cs, warps, s, cfg, attr);
   if (st != VEF_OK) return st;
   KTimer kt(B.meshes[C.probs[0]], VEF_K_SWEEP, s);
   VEF_CUDA_TRY(cudaLaunchKernelEx(&cfg, sweep_batch_kernel<P, double, 0>, (const SweepArgs<double>*)C.tab_dev,
