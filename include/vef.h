@@ -70,7 +70,8 @@ typedef enum {
   VEF_ERR_INVALID_ARG = 1,
   VEF_ERR_CUDA = 2,
   VEF_ERR_OOM = 3,
-  VEF_ERR_TIMEOUT = 4,            /* a bounded device-side wait (staging copy) gave up */
+  VEF_ERR_TIMEOUT = 4,            /* a bounded device-side wait (a staging copy, a band of the
+                                     fused apply, a grid barrier of the HRT solve) gave up */
   VEF_ERR_NOT_CONVERGED = 5,      /* an inner or defect-correction iteration hit its cap */
   VEF_ERR_NONPOSITIVE_DENOM = 6,  /* sum_d w_d psi_d <= 1e-300 at a closure point (NaN written) */
   VEF_ERR_NOT_IMPLEMENTED = 7,
@@ -323,9 +324,11 @@ vef_status vef_batch_tune(vef_batch batch, void* stream, int* tiles_out);
  *   a + (p+2) b, then y part a + (p+1) b), lambda [device] [faces][p+1] or NULL (interior
  *   faces: vertical ones first, j (nx-1) + i, then horizontal, (nx-1) ny + j nx + i).
  * Synchronises `stream` (the Krylov scalars stay on the device; the host reads the
- * convergence state back every 16 iterations).  Uses the handle's
- * scratch.  Errors: VEF_ERR_INVALID_ARG, VEF_ERR_NOT_CONVERGED (tolerance not reached in
- * max_iter iterations, or a singular local system). */
+ * convergence state back every 256 iterations).  The iterations run in a cooperative launch
+ * of at most one CTA per SM (a context limited to fewer SMs gets a smaller one).  Uses the
+ * handle's scratch.  Errors: VEF_ERR_INVALID_ARG, VEF_ERR_NOT_CONVERGED (tolerance not reached
+ * in max_iter iterations, or a singular local system), VEF_ERR_TIMEOUT (a grid barrier's wait
+ * ran out, or a timeout was pending); a failed call clears the handle's status word too. */
 typedef struct {
   int iterations;          /* BiCGStab iterations of the multiplier system */
   double rel_residual;     /* final ||r - H lambda||_2 / ||r||_2 */
@@ -431,6 +434,12 @@ vef_status vef_schedule_host(int nx, int ny, int p, const double* nds, const dou
  * polls in 1..2^24, else VEF_ERR_INVALID_ARG (checked before any CUDA call).  Allocates and
  * frees 8 bytes of device memory. */
 vef_status vef_wait_selftest(int kind, int satisfied, long long polls, void* stream);
+
+/* The same for the grid barrier of the HRT multiplier solve, in a one-CTA kernel at which one
+ * arrival is awaited (satisfied != 0 -> VEF_OK) or two (satisfied == 0: VEF_ERR_TIMEOUT after
+ * `polls` polls).  polls in 1..2^24, else VEF_ERR_INVALID_ARG (checked before any CUDA call).
+ * Allocates and frees 8 bytes of device memory. */
+vef_status vef_grid_wait_selftest(int satisfied, long long polls, void* stream);
 
 /* The elimination pivots' reciprocal (an approximate reciprocal refined by two
  * Newton-Raphson steps; FP32: the correctly rounded reciprocal) against the correctly

@@ -39,8 +39,9 @@ VEF_STATUS_BOUNDS = 16
 # every symbol include/vef.h declares
 EXPORTS = ("vef_mesh_create", "vef_mesh_destroy", "vef_mesh_query", "vef_mesh_sync", "vef_sweep",
            "vef_moments", "vef_source_iterate", "vef_adjoint_sweep", "vef_profile",
-           "vef_profile_read", "vef_measure_fma_peak", "vef_wait_selftest", "vef_eddington_noalloc",
-           "vef_batch_create", "vef_batch_destroy", "vef_batch_sweep", "vef_batch_tune",
+           "vef_profile_read", "vef_measure_fma_peak", "vef_wait_selftest",
+           "vef_grid_wait_selftest", "vef_eddington_noalloc", "vef_batch_create", "vef_batch_destroy",
+           "vef_batch_sweep", "vef_batch_tune",
            "vef_region_weights", "vef_schedule_host", "vef_mesh_inject_status", "vef_hrt_solve",
            "vef_vef_iterate", "vef_build_checked", "vef_rcp_selftest",
            "vef_status_string", "vef_last_error")
@@ -118,6 +119,7 @@ def _declare(lib):
     lib.vef_profile_read.argtypes = [P, ctypes.POINTER(VefKernelStat)]
     lib.vef_measure_fma_peak.argtypes = [I, ctypes.POINTER(ctypes.c_double)]
     lib.vef_wait_selftest.argtypes = [I, I, ctypes.c_longlong, P]
+    lib.vef_grid_wait_selftest.argtypes = [I, ctypes.c_longlong, P]
     lib.vef_schedule_host.argtypes = [I, I, I, P, P, I, P, P, P, P]
     lib.vef_eddington_noalloc.argtypes = [P, P, P, I, ctypes.c_longlong, I, P, P]
     PP = ctypes.POINTER(ctypes.c_void_p)
@@ -134,7 +136,7 @@ def _declare(lib):
     for name in ("vef_mesh_create", "vef_mesh_destroy", "vef_mesh_query", "vef_mesh_sync",
                  "vef_sweep", "vef_moments", "vef_source_iterate", "vef_adjoint_sweep",
                  "vef_profile", "vef_profile_read", "vef_measure_fma_peak", "vef_wait_selftest",
-                 "vef_eddington_noalloc", "vef_batch_create", "vef_batch_destroy",
+                 "vef_grid_wait_selftest", "vef_eddington_noalloc", "vef_batch_create", "vef_batch_destroy",
                  "vef_batch_sweep", "vef_batch_tune", "vef_region_weights", "vef_schedule_host",
                  "vef_mesh_inject_status", "vef_hrt_solve", "vef_vef_iterate"):
         getattr(lib, name).restype = I

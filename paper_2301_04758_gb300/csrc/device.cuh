@@ -180,6 +180,34 @@ __device__ __forceinline__ int ld_acquire_gpu(const int* p) {
   asm volatile("ld.acquire.gpu.global.b32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
   return v;
 }
+// Barrier over the CTAs of a cooperative launch (all resident), every thread of each: `arrivals`
+// CTAs arrive at it, counted up in *count from zero over the launch, epoch being the count
+// that completes it.  Bounded: after `polls` polls the timeout bit is set and the barrier gives
+// up, and so it does, looked up at the first poll and every 16, once the status word carries a
+// timeout (another CTA's wait ran out, or the call began with an uncollected one).  Returns whether it completed;
+// a CTA that gets false leaves, and the others do as their waits end.
+__device__ __forceinline__ bool grid_barrier(unsigned* count, unsigned& epoch, unsigned arrivals, unsigned polls,
+                                             unsigned int* status) {
+  __shared__ int ok;
+  epoch += arrivals;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    atomicAdd(count, 1u);
+    for (unsigned n = 0;;) {
+      const unsigned bits = (n & 15u) == 0 ? *(const volatile unsigned int*)status : 0;
+      const bool done = (unsigned)ld_acquire_gpu((const int*)count) >= epoch;
+      ok = done;
+      if (done || (bits & kDevTimeout)) break;
+      if (++n >= polls) {
+        atomicOr(status, kDevTimeout);
+        break;
+      }
+    }
+  }
+  __syncthreads();
+  return ok != 0;
+}
 // order this thread's earlier generic-proxy view of global memory before later bulk copies
 __device__ __forceinline__ void fence_proxy_async_global() {
   asm volatile("fence.proxy.async.global;" ::: "memory");

@@ -72,6 +72,19 @@ __global__ void wait_selftest_kernel(int kind, int satisfied, uint32_t polls, co
   if (n >= polls) atomicOr(status, kDevTimeout);
 }
 
+// The same for the grid barrier of the HRT multiplier solve: one CTA arrives where `arrivals` are
+// awaited, so that the wait ends at once (1) or runs out (2).
+__global__ void grid_wait_selftest_kernel(unsigned arrivals, unsigned polls, unsigned* count, unsigned int* status) {
+  unsigned epoch = 0;
+  grid_barrier(count, epoch, arrivals, polls, status);
+}
+
+static vef_status wait_selftest_result(unsigned int bits) {
+  if (!(bits & kDevTimeout)) return VEF_OK;
+  set_last_error("the bounded wait ran out and reported a timeout");
+  return VEF_ERR_TIMEOUT;
+}
+
 }  // namespace vef
 
 extern "C" vef_status vef_wait_selftest(int kind, int satisfied, long long polls, void* stream) {
@@ -93,8 +106,26 @@ extern "C" vef_status vef_wait_selftest(int kind, int satisfied, long long polls
   if (err == cudaSuccess) err = cudaStreamSynchronize(s);
   cudaFree(buf);
   if (err != cudaSuccess) return cuda_fail(err, "wait self-test");
-  if (bits & kDevTimeout) { set_last_error("the bounded wait ran out and reported a timeout"); return VEF_ERR_TIMEOUT; }
-  return VEF_OK;
+  return wait_selftest_result(bits);
+}
+
+extern "C" vef_status vef_grid_wait_selftest(int satisfied, long long polls, void* stream) {
+  using namespace vef;
+  if (polls < 1 || polls > (1LL << 24)) { set_last_error("polls must be in 1..2^24"); return VEF_ERR_INVALID_ARG; }
+  cudaStream_t s = (cudaStream_t)stream;
+  unsigned* buf = nullptr;   // [0] the arrival count, [1] the status word
+  VEF_CUDA_TRY(cudaMalloc(&buf, 2 * sizeof(unsigned)));
+  cudaError_t err = cudaMemsetAsync(buf, 0, 2 * sizeof(unsigned), s);
+  if (err == cudaSuccess) {
+    grid_wait_selftest_kernel<<<1, 64, 0, s>>>(satisfied ? 1u : 2u, (unsigned)polls, buf, buf + 1);
+    err = cudaGetLastError();
+  }
+  unsigned int bits = 0;
+  if (err == cudaSuccess) err = cudaMemcpyAsync(&bits, buf + 1, sizeof(bits), cudaMemcpyDeviceToHost, s);
+  if (err == cudaSuccess) err = cudaStreamSynchronize(s);
+  cudaFree(buf);
+  if (err != cudaSuccess) return cuda_fail(err, "grid wait self-test");
+  return wait_selftest_result(bits);
 }
 
 extern "C" vef_status vef_measure_fma_peak(int precision, double* flops_per_s) {

@@ -827,7 +827,7 @@ __global__ void hrt_recover_kernel(long long E, int nx, int ny, const double* __
 constexpr int kKT = 512, kCheck = 256;   // threads per CTA; iterations per launch
 enum { kDotRR = 0, kDotRV = 1, kDotRS = 2, kDotTS = 3, kDotTT = 4, kDotRT = 5, kNumDots = 6 };
 constexpr size_t kTileSmemMax = 160 * 1024;
-constexpr unsigned kGridPolls = 1u << 22;   // a poll takes ~0.3 us or more: a second or so
+constexpr unsigned kGridPolls = 1u << 22;   // a poll takes 0.23 us (vef_grid_wait_selftest), so about a second
 
 struct KState {
   int done;      // 1: converged, 2: breakdown
@@ -1223,24 +1223,8 @@ __device__ __forceinline__ int kry_dof(const Kry& k, int side, int i, int j, int
   return (side == 0 ? j * (k.nx - 1) + i - 1 : (k.nx - 1) * k.ny + (j - 1) * k.nx + i) * (P + 1) + tt;
 }
 
-// Grid barrier of a cooperative launch (all CTAs resident): arrivals are counted up from zero
-// over the launch.  Bounded: when the polls run out the timeout bit is set and every CTA that
-// sees the count short leaves.  Returns whether the barrier completed.
 __device__ __forceinline__ bool kry_barrier(KState* st, unsigned& epoch, unsigned int* status) {
-  __shared__ int ok;
-  epoch += gridDim.x;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    __threadfence();
-    atomicAdd(&st->bar, 1u);
-    unsigned n = 0;
-    while ((unsigned)ld_acquire_gpu((const int*)&st->bar) < epoch && ++n < kGridPolls) {
-    }
-    ok = n < kGridPolls;
-    if (n >= kGridPolls) atomicOr(status, kDevTimeout);
-  }
-  __syncthreads();
-  return ok != 0;
+  return grid_barrier(&st->bar, epoch, gridDim.x, kGridPolls, status);
 }
 
 // The scalars of the iteration, kept by thread 0 of every CTA (the same values in the same
@@ -1885,7 +1869,9 @@ static vef_status hrt_run(Mesh& M, const HrtIn& in, double tol, int max_iter, do
       it += n;
       if (!hs.done && hs.base != it) {   // a grid barrier's wait ran out: the launch left early
         st = collect_status(M, s, nullptr);
-        return st != VEF_OK ? st : VEF_ERR_TIMEOUT;
+        if (st != VEF_OK && st != VEF_ERR_TIMEOUT) return st;
+        set_last_error("a grid barrier of the HRT multiplier solve gave up (a bounded device-side wait ran out)");
+        return VEF_ERR_TIMEOUT;
       }
     }
     if (hs.done) it = hs.iters;

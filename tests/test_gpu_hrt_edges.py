@@ -92,3 +92,31 @@ def test_dot_products_near_the_end_of_the_range(lib):
     phi, J, lam, info = _solve(Mesh(2, 1, 1, p, 0.0), big, tol=1e-13)
     for got, key in ((phi, "phi"), (J, "J"), (lam, "lam")):
         assert rel(got / scale, v[key]) < 1e-11, info
+
+
+def test_grid_barrier_gives_up(lib):
+    """The grid barrier's wait runs out when an arrival is missing, with the status for it, and a
+    solve that begins with a timeout pending leaves at its first barriers, says so and lets the
+    next one succeed."""
+    from paper_2301_04758_gb300 import _lib
+    from paper_2301_04758_gb300.api import Mesh
+    polls = 1 << 12
+    assert lib.vef_grid_wait_selftest(1, polls, None) == _lib.VEF_OK
+    t = time.perf_counter()
+    st = lib.vef_grid_wait_selftest(0, polls, None)
+    elapsed = time.perf_counter() - t
+    print(f"{polls} polls ran out in {elapsed * 1e3:.2f} ms ({elapsed / polls * 1e9:.0f} ns per poll, launch included)")
+    assert st == _lib.VEF_ERR_TIMEOUT and elapsed < 5.0
+    assert lib.vef_grid_wait_selftest(0, 0, None) == _lib.VEF_ERR_INVALID_ARG
+    assert lib.vef_grid_wait_selftest(0, (1 << 24) + 1, None) == _lib.VEF_ERR_INVALID_ARG
+    n, p = 48, 2
+    v = exact_problem(n, n, p, 860)
+    mesh = Mesh(n, n, 1, p, 0.0)
+    _solve(mesh, v, tol=1e-13)
+    assert lib.vef_mesh_inject_status(mesh.handle, _lib.VEF_STATUS_TIMEOUT, None) == _lib.VEF_OK
+    t = time.perf_counter()
+    with pytest.raises(_lib.VefError, match="grid barrier") as err:
+        _solve(mesh, v, tol=1e-13)
+    assert err.value.status == _lib.VEF_ERR_TIMEOUT and time.perf_counter() - t < 0.5
+    phi, J, lam, _ = _solve(mesh, v, tol=1e-13)
+    assert rel(phi, v["phi"]) < 1e-9 and rel(J, v["J"]) < 1e-9 and rel(lam, v["lam"]) < 1e-9
