@@ -808,7 +808,7 @@ __global__ void hrt_recover_kernel(long long E, int nx, int ny, const double* __
 // ---- the multiplier system's Krylov solve: BiCGStab (van der Vorst) with the two-level
 // Schwarz preconditioner (the element patches above and the coarse space below) as one
 // cooperative kernel, kry_solve_kernel.  The mesh is cut into tiles of whole elements, each
-// inside one coarse cell; a CTA takes a tile (or several) and owns the multipliers of the
+// inside one coarse cell (kry_cut); a CTA takes a tile (or several) and owns the multipliers of the
 // left and bottom faces of its elements.  Vectors that other tiles read live in global
 // memory and are read past L1; a phase's own intermediate (the vector the element patches or
 // the matrix act on, with its halo) sits in shared memory.  One iteration is four phases,
@@ -827,6 +827,7 @@ __global__ void hrt_recover_kernel(long long E, int nx, int ny, const double* __
 constexpr int kKT = 512, kCheck = 256;   // threads per CTA; iterations per launch
 enum { kDotRR = 0, kDotRV = 1, kDotRS = 2, kDotTS = 3, kDotTT = 4, kDotRT = 5, kNumDots = 6 };
 constexpr size_t kTileSmemMax = 160 * 1024;
+constexpr int kTileMin = 16;   // elements
 constexpr unsigned kGridPolls = 1u << 22;   // a poll takes 0.23 us (vef_grid_wait_selftest), so about a second
 
 struct KState {
@@ -1735,6 +1736,31 @@ __global__ void __launch_bounds__(kKT, 1) kry_solve_kernel(Kry k, int n, int che
 
 static inline unsigned nblk(long long n, int bs) { return (unsigned)((n + bs - 1) / bs); }
 
+// The tiles of the Krylov kernel: a coarse cell each, cut along its longer side while its staged
+// vector with its halo does not fit a CTA's shared memory, and on while every tile still has an
+// SM of its own and more than kTileMin elements.  The second rule serves strips, whose coarse grid
+// has few cells: whole solves 10000 x 1 Q2 12.7 -> 5.4 ms, 1000 x 4 3.6 -> 2.7, 500 x 5 2.5 -> 2.2;
+// with a limit of 8 elements 100 x 3 Q3 takes 1.29 ms instead of 1.22 (shorter tiles, the same
+// barriers), with 64 1000 x 4 takes 3.1.  A mesh of 11 x 11 cells is cut for shared memory only.
+template <typename Fits>
+static void kry_cut(Kry& k, int sms, Fits fits) {
+  k.sx = k.sy = 1;
+  k.tw = k.cx;
+  k.th = k.cy;
+  for (;;) {
+    const bool wide = k.tw >= k.th;
+    // the fewest parts shorter than now, of even length: none is empty in a whole cell
+    const int sx = wide && k.tw > 1 ? (k.cx + k.tw - 2) / (k.tw - 1) : k.sx;
+    const int sy = !wide && k.th > 1 ? (k.cy + k.th - 2) / (k.th - 1) : k.sy;
+    const int w = (k.cx + sx - 1) / sx, h = (k.cy + sy - 1) / sy;
+    if (fits() && ((long long)k.ncx * k.ncy * sx * sy > sms || k.tw * k.th <= kTileMin)) return;
+    k.tw = w;
+    k.th = h;
+    k.sx = sx;
+    k.sy = sy;
+  }
+}
+
 template <int P>
 static vef_status hrt_run(Mesh& M, const HrtIn& in, double tol, int max_iter, double* phi, double* J,
                           double* lambda, vef_hrt_info* info, cudaStream_t s, bool& launched) {
@@ -1773,14 +1799,11 @@ static vef_status hrt_run(Mesh& M, const HrtIn& in, double tol, int max_iter, do
     double gw[kMaxP + 1];
     gauss_legendre(P + 1, k.gl, gw);
   }
-  // tiles of the Krylov kernel: a coarse cell each, cut further while a tile's staged vector
-  // with its halo would not fit a CTA's shared memory
+  int dev = 0, sms = 0, inv_per_sm = 0;
+  VEF_CUDA_TRY(cudaGetDevice(&dev));
+  VEF_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   auto tile_smem = [&] { return (size_t)(k.tw + 2) * (k.th + 2) * 2 * S::NL * sizeof(double); };
-  for (k.sx = k.sy = 1;; ++k.sx, ++k.sy) {
-    k.tw = (k.cx + k.sx - 1) / k.sx;
-    k.th = (k.cy + k.sy - 1) / k.sy;
-    if (tile_smem() <= kTileSmemMax) break;
-  }
+  kry_cut(k, sms, [&] { return tile_smem() <= kTileSmemMax; });
   k.ntiles = k.ncx * k.ncy * k.sx * k.sy;
   const size_t total = per_e * E + 10 * vec + (size_t)(S::NL4 * S::NL4 + S::NL4) * E +
                        (size_t)nc * nc + 16 * (size_t)k.ncx * k.ncy + 4 * (size_t)k.ntiles + 2 * vec +
@@ -1817,9 +1840,6 @@ static vef_status hrt_run(Mesh& M, const HrtIn& in, double tol, int max_iter, do
   if ((st = allow_dynamic_smem<hrt_local_kernel<P>>()) != VEF_OK) return st;
   if ((st = allow_dynamic_smem<hrt_invert_kernel<P>>()) != VEF_OK) return st;
   if ((st = allow_dynamic_smem<hrt_coarse_pivot_kernel>()) != VEF_OK) return st;
-  int dev = 0, sms = 0, inv_per_sm = 0;
-  VEF_CUDA_TRY(cudaGetDevice(&dev));
-  VEF_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   VEF_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&inv_per_sm, hrt_invert_kernel<P>, HrtInvShape<P>::T, ismem));
   launched = true;
   {

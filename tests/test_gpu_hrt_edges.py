@@ -120,3 +120,48 @@ def test_grid_barrier_gives_up(lib):
     assert err.value.status == _lib.VEF_ERR_TIMEOUT and time.perf_counter() - t < 0.5
     phi, J, lam, _ = _solve(mesh, v, tol=1e-13)
     assert rel(phi, v["phi"]) < 1e-9 and rel(J, v["J"]) < 1e-9 and rel(lam, v["lam"]) < 1e-9
+
+
+@pytest.mark.parametrize("nx,ny,p,least", [(1090, 1, 2, 0), (1, 1090, 3, 0), (500, 5, 1, 0), (12600, 7, 2, 0), (7, 7500, 4, 0),
+                                           (640, 640, 2, 257)],
+                         ids=["cut_with_empty", "cut_upright", "cut_cells", "tiles_per_cta", "tiles_per_cta_upright",
+                              "cut_square_two_launches"])
+def test_krylov_tiles_of_large_and_long_meshes(lib, nx, ny, p, least):
+    """Cells of the coarse grid cut into several tiles: because a strip has few cells (at 1090
+    the last cell's last tile is empty), because the staged vector would not fit (then more tiles
+    than CTAs, each taking its share), and more iterations than one launch runs.  phi, J and the
+    multipliers against the exact solution; absorption keeps H's condition below about 1e3 per
+    coarse cell, so a relative residual of 1e-12 leaves 1e-9."""
+    from paper_2301_04758_gb300.api import Mesh
+    scale = max(nx, ny) / 10 if min(nx, ny) < 100 else 1.0
+    v = exact_problem(nx, ny, p, 870, sigma=(0.5 * scale, 5.0 * scale))
+    phi, J, lam, info = _solve(Mesh(nx, ny, 1, p, 0.0), v, tol=1e-12)
+    assert info["iterations"] >= least and info["multipliers"] == lam.size, info
+    assert rel(phi, v["phi"]) < 1e-9 and rel(J, v["J"]) < 1e-9 and rel(lam, v["lam"]) < 1e-9, info
+
+
+def test_a_strip_keeps_the_device_busy(lib):
+    """An iteration on 10000 x 1 elements takes less than twice one on 100 x 100 (3.7 times when
+    each of the strip's eleven coarse cells was one CTA's)."""
+    from paper_2301_04758_gb300.api import Mesh
+    import torch
+
+    def per_iteration(nx, ny):
+        scale = max(nx, ny) / 10
+        v = exact_problem(nx, ny, 2, 880, sigma=(0.5 * scale, 5.0 * scale))
+        mesh = Mesh(nx, ny, 1, 2, 0.0)
+        args = [dev(v[k]) for k in ("sigma_t", "sigma_s", "phi_tr", "P_tr", "Eb", "Jin", "Q0", "Q1")]
+
+        def run(its):
+            times = []
+            for _ in range(7):
+                torch.cuda.synchronize()
+                t = time.perf_counter()
+                info = mesh.hrt_solve(*args, tol=1e-15, max_iter=its, check=False)[3]
+                times.append(time.perf_counter() - t)
+                assert info["iterations"] == its
+            return sorted(times)[3]
+        return (run(34) - run(4)) / 30
+    strip, square = per_iteration(10000, 1), per_iteration(100, 100)
+    print(f"strip {strip * 1e6:.1f} us, square {square * 1e6:.1f} us per iteration")
+    assert strip < 2.0 * square
