@@ -1621,7 +1621,7 @@ __global__ void __launch_bounds__(kKT, 1) kry_solve_kernel(Kry k, int n, int che
               k.rh[m] = ri;
               k.x[m] = 0.0;
             } else {
-              k.x[m] = fma(omega, k.sh[m], fma(alpha, k.ph[m], k.x[m]));
+              k.x[m] += fma(omega, k.sh[m], alpha * k.ph[m]);   // one rounding at the size of x
               k.r[m] = ri;
             }
             pn[m] = pm;

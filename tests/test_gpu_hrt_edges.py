@@ -165,3 +165,30 @@ def test_a_strip_keeps_the_device_busy(lib):
     strip, square = per_iteration(10000, 1), per_iteration(100, 100)
     print(f"strip {strip * 1e6:.1f} us, square {square * 1e6:.1f} us per iteration")
     assert strip < 2.0 * square
+
+
+# pairs of sizes and two seeds each: errors of single solves scatter by a factor of ten
+_SIZES = [(13, 17), (19, 23), (26, 31), (40, 40), (33, 29), (45, 37), (22, 41), (51, 14), (28, 28), (37, 43), (16, 16),
+          (32, 32), (24, 36), (30, 50)]
+
+
+def _mean_error(key, sigma, scatter, p=1):
+    """Geometric mean over the sizes of the relative error of phi or J, iterated until the
+    residual no longer falls."""
+    from paper_2301_04758_gb300.api import Mesh
+    errors = []
+    for nx, ny in _SIZES:
+        for seed in (100, 101):
+            v = exact_problem(nx, ny, p, seed, sigma, scatter)
+            phi, J, _, _ = _solve(Mesh(nx, ny, 1, p, 0.0), v, tol=1e-15, max_iter=400, check=False)
+            errors.append(rel({"phi": phi, "J": J}[key], v[key]))
+    return np.exp(np.mean(np.log(errors)))
+
+
+@pytest.mark.parametrize("sigma,scatter,limit", [((1e-3, 1e-2), (0.5, 0.9), 4.6e-11), ((0.5, 5.0), (0.3, 0.95), 8.4e-14),
+                                                 ((0.5, 5.0), (1.0, 1.0), 8.2e-14)], ids=["thin", "mid", "scattering"])
+def test_the_multiplier_update_rounds_once(lib, sigma, scatter, limit):
+    """J's mean error against the exact solution stays within an eighth of what it is with one
+    rounding at the size of lambda per iteration (4.1e-11, 7.5e-14, 7.3e-14; with two, by a
+    chain of multiply-adds, 5.1e-11, 9.2e-14, 9.4e-14)."""
+    assert _mean_error("J", sigma, scatter) < limit
