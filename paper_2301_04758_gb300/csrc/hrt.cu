@@ -207,10 +207,18 @@ static void make_hrt_ref(const HrtTab& t, HrtRef<P>& o) {
       }
     }
   }
+  // D and C1 round the same way on every element, and phi collects what breaks the balance of
+  // D's columns with C1's: the order of these products is kept (another one tripled phi's error
+  // at p = 1 in thin media)
   for (int r = 0; r < N; ++r)
     for (int c = 0; c < NJ; ++c) {
       double s = 0.0;
-      for (int pt = 0; pt < NQ2; ++pt) s += o.w[pt] * o.bt[pt][r] * (c < S::NX ? o.r0[pt][c] : o.r1[pt][c]);
+      for (int k2 = 0; k2 < NQ; ++k2)
+        for (int k1 = 0; k1 < NQ; ++k1) {
+          double v, dx, dy;
+          rt_ref<P>(t, c, k1, k2, v, dx, dy);
+          s += t.w[k1] * t.w[k2] * t.dg[r % Q][k1] * t.dg[r / Q][k2] * (c < S::NX ? dx : dy);
+        }
       o.D[r * NJ + c] = s;
     }
   for (int f = 0; f < 4; ++f) {
@@ -218,7 +226,7 @@ static void make_hrt_ref(const HrtTab& t, HrtRef<P>& o) {
     for (int tt = 0; tt < NL; ++tt)
       for (int a = 0; a < NJ; ++a) {
         double s = 0.0;
-        for (int k = 0; k < NQ; ++k) s += t.w[k] * o.c2[f * NL + tt][k][a] * (a < S::NX ? n0 : n1);
+        for (int k = 0; k < NQ; ++k) s += t.w[k] * t.op[tt][k] * (o.fv[f * NQ + k][a] * (a < S::NX ? n0 : n1));
         o.C1[(f * NL + tt) * NJ + a] = s;
       }
   }
