@@ -852,8 +852,7 @@ static_assert(sizeof(KState) % sizeof(double) == 0, "KState is carved from a dou
 
 struct Kry {
   int nx, ny;
-  long long nfaces, nl;
-  long long E;
+  long long nl;
   const double* He;
   const double* Pinv;   // [E][4 (p+1)][4 (p+1)] element-patch inverses of the preconditioner
   double* z;            // [E][4 (p+1)] the preconditioner's element results
@@ -1243,7 +1242,7 @@ __device__ __forceinline__ bool kry_barrier(KState* st, unsigned& epoch, unsigne
 struct KryScal {
   double dot[4];
   double rho, rho_new, alpha, omega, beta, bb, rr, tol2;
-  int it, done, iters, brk;
+  int done, iters, brk;
 };
 
 // a / b to within two ulp: the approximate reciprocal refined by two Newton-Raphson steps
@@ -1828,14 +1827,13 @@ static vef_status hrt_run(Mesh& M, const HrtIn& in, double tol, int max_iter, do
   double* f = take((size_t)S::N * E);
   double* He = take((size_t)S::NL4 * S::NL4 * E);
   double* re = take((size_t)S::NL4 * E);
-  k.nx = M.nx; k.ny = M.ny; k.nfaces = nfaces; k.nl = nl; k.He = He;
+  k.nx = M.nx; k.ny = M.ny; k.nl = nl; k.He = He;
   k.x = lambda && nl > 0 ? lambda : take(vec);
   k.r = take(vec); k.rh = take(vec); k.p[0] = take(vec); k.p[1] = take(vec); k.v = take(vec); k.s = take(vec);
   k.t = take(vec); k.ph = take(vec); k.sh = take(vec);
   double* Pinv = take((size_t)S::NL4 * S::NL4 * E);
   k.Pinv = Pinv;
   k.z = take((size_t)S::NL4 * E);
-  k.E = E;
   k.A0 = take((size_t)nc * nc);
   k.pc = take((size_t)4 * k.ntiles);
   double* Acell = take((size_t)16 * k.ncx * k.ncy);
