@@ -829,9 +829,10 @@ __global__ void hrt_recover_kernel(long long E, int nx, int ny, const double* __
 //   D  s_hat as in B; t = H s_hat; t.s, t.t, r_hat.t
 // (rho of the next iteration is r_hat.s - omega r_hat.t, so it needs no barrier of its own).
 // Every dot product is summed in a fixed order (per tile, then over the tiles), so the
-// iteration is deterministic.  The waits at the barriers are bounded.  FP64 issue and the
-// barriers bound it: 67 us per iteration at 128^2 Q2 and about 30 at 24 x 20 Q3, where 11
-// launches replayed from a graph took 78 and 62.
+// iteration is deterministic.  The waits at the barriers are bounded.  66 us per iteration at
+// 128^2 Q2, where the FP64 pipe of the 121 SMs with a tile is busy 65 % of the time and shared
+// memory's latency and the block and grid barriers take the rest; about 30 at 24 x 20 Q3, mostly
+// barriers.  11 launches replayed from a graph took 78 and 62.
 constexpr int kKT = 512, kCheck = 256;   // threads per CTA; iterations per launch
 enum { kDotRR = 0, kDotRV = 1, kDotRS = 2, kDotTS = 3, kDotTT = 4, kDotRT = 5, kNumDots = 6 };
 constexpr size_t kTileSmemMax = 160 * 1024;
