@@ -360,7 +360,7 @@ factor_pivot_kernel(long long nmem, const uint32_t* __restrict__ code, const uin
 // column goes last), so that the steps run in a loop: unrolled, the elimination is some 60 KB
 // of instructions at p = 3 and 130 KB at p = 4, and warps out of step with one another wait for
 // instruction fetch (256^2 Q3 S12 call: 73.2 ms unrolled, 67.0 ms turned).
-template <int P, typename T> struct ElemShape;
+template <int P, typename T, bool FEW = false> struct ElemShape;
 // EPC elements per CTA: at p = 3 in FP64 a warp holds 8 tasks, and the level-symmetric sets
 // have D = 4 (mod 8) directions for S4 and S12, so one element per CTA would leave half a
 // warp of padding tasks computing; two elements per CTA fill every warp (2 D = 0 mod 8).
@@ -373,6 +373,12 @@ template <int P, typename T> struct ElemShape;
 template <> struct ElemShape<3, double> { static constexpr int RPL = 4, LPU = 4, EPC = 2, NW = 1, MINB = 1; };
 template <> struct ElemShape<3, float> { static constexpr int RPL = 2, LPU = 8, EPC = 4, NW = 4, MINB = 6; };
 template <> struct ElemShape<4, float> { static constexpr int RPL = 2, LPU = 13, EPC = 1, NW = 4, MINB = 1; };
+// FEW: grids in FP64 whose warps all run at once (factor_few).  A warp's FP64 instructions take its
+// SM's quarter 64 cycles each, so there the rows on a lane set a round's time and two per lane beat
+// four: factorisation of 8^2 Q4 S4 174 -> 88 us (146 with two rows, four warps and no parts), Q3
+// 80 -> 51 us (78).
+template <> struct ElemShape<3, double, true> { static constexpr int RPL = 2, LPU = 8, EPC = 1, NW = 1, MINB = 1; };
+template <> struct ElemShape<4, double, true> { static constexpr int RPL = 2, LPU = 13, EPC = 1, NW = 1, MINB = 1; };
 
 // an element's (or CTA's elements') rounds are spread over `parts` CTAs: CTA blockIdx.x takes
 // [r0, r1)
@@ -386,17 +392,28 @@ __device__ __forceinline__ void part_rounds(int rounds, int parts, int& r0, int&
 // element for too few rounds.  Whole call without and with parts: 23^2 Q3 S4 0.417 -> 0.313 ms,
 // 64^2 Q3 S6 2.17 -> 2.07, 61 x 47 Q4 S6 5.20 -> 4.70, 64^2 Q4 S12 17.6 -> 16.0; the grids that
 // give six waves by themselves (256^2 Q3 S12) take one part.
-constexpr int kPartWaves = 6;
-static int factor_parts(long long groups, int rounds) {
+constexpr int kPartWaves = 6, kWarpsPerSm = 8;
+static int sm_count() {
   int dev = 0, sms = 1;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const long long want = (long long)sms * 8 * kPartWaves;
+  return sms;
+}
+static int factor_parts(long long groups, int rounds) {
+  const long long want = (long long)sm_count() * kWarpsPerSm * kPartWaves;
   return (int)std::max(1LL, std::min<long long>(rounds, (want + groups - 1) / groups));
 }
+// whether E elements' rounds in the FEW shape, one warp each, are at most kWarpsPerSm per SM.  At
+// 6.6 per SM (10^2 Q3 S8) it takes 70 us and the other shape 82, at 7.7 (14^2 Q4 S4) 140 and 177; at
+// 8.4 (8^2 Q4 S8) 207 and 167, at 15 (8^2 Q3 S16) 137 and 125.
+template <int P>
+static bool factor_few(long long E, int D) {
+  constexpr int UPW = 32 / ElemShape<P, double, true>::LPU;
+  return E * ((D + UPW - 1) / UPW) <= (long long)sm_count() * kWarpsPerSm;
+}
 
-template <int P, typename T, bool Y>
-__global__ void __launch_bounds__(32 * ElemShape<P, T>::NW, ElemShape<P, T>::MINB)
+template <int P, typename T, bool Y, bool FEW>
+__global__ void __launch_bounds__(32 * ElemShape<P, T, FEW>::NW, ElemShape<P, T, FEW>::MINB)
 factor_elem_kernel(int D, long long E, const int* __restrict__ member_of, const uint16_t* __restrict__ finfo,
                    const double* __restrict__ omega, const double* __restrict__ sigma_t,
                    const T* __restrict__ Mm, const T* __restrict__ Gxm, const T* __restrict__ Gym,
@@ -404,7 +421,8 @@ factor_elem_kernel(int D, long long E, const int* __restrict__ member_of, const 
                    T* __restrict__ rec, unsigned int* status, unsigned int* piv_count,
                    unsigned int* piv_list, int force_pivot, RhsArgs<T> rhs, int parts) {
   constexpr int Q = P + 1, N = Q * Q, NQ = P + 2;
-  constexpr int RPL = ElemShape<P, T>::RPL, LPU = ElemShape<P, T>::LPU, UPW = 32 / LPU, EPC = ElemShape<P, T>::EPC;
+  using Sh = ElemShape<P, T, FEW>;
+  constexpr int RPL = Sh::RPL, LPU = Sh::LPU, UPW = 32 / LPU, EPC = Sh::EPC;
   constexpr int LD = N + 1;                  // padded shared-memory row stride
   constexpr int CPL = (Q * Q + LPU - 1) / LPU;   // inflow-coupling entries computed per lane
   constexpr unsigned FULL = 0xffffffffu;
@@ -413,7 +431,7 @@ factor_elem_kernel(int D, long long E, const int* __restrict__ member_of, const 
   __shared__ T sN[EPC][4 * NQ * 2];
   __shared__ T sLL[Q][Q][NQ];          // l_a(s_k) l_t(s_k): face basis products
   __shared__ T sW[NQ];                 // face Gauss weights
-  __shared__ T sC[ElemShape<P, T>::NW][UPW][4][NQ];   // per warp and task: w_k Omega . (n ds)_k of each face
+  __shared__ T sC[Sh::NW][UPW][4][NQ];   // per warp and task: w_k Omega . (n ds)_k of each face
   const long long e0 = (long long)(blockIdx.x / parts) * EPC;
   const int ne = (int)min((long long)EPC, E - e0);   // elements of this CTA
   const int tid = threadIdx.x;
@@ -1380,22 +1398,30 @@ static vef_status launch_factor(Mesh& M, Schedule& S, const double* sigma_t, boo
   VEF_CUDA_TRY(cudaMemsetAsync(piv_count, 0, sizeof(unsigned int), stream));
   {
   KTimer kt(&M, VEF_K_FACTOR, stream);
-  if constexpr (P == 4 && sizeof(T) == 8) {
-    auto kern = rhs ? factor_elem4_kernel<true> : factor_elem4_kernel<false>;
-    const int parts = factor_parts(M.E, (S.D + 4) / 5);
-    kern<<<(unsigned)(M.E * parts), 32, 0, stream>>>(S.D, M.E, S.member_of, S.faceinfo, S.omega_dev, sigma_t, Mm, Gx, Gy, nds,
-                                           make_facetab<T>(M.tab), M.nx, M.ny, S.members, (T*)*recp, M.dev_status,
-                                           piv_count, S.pivot_list, force_pivot, ra, parts);
-  } else if constexpr (P >= 3) {
-    constexpr int UPW = 32 / ElemShape<P, T>::LPU, EPC = ElemShape<P, T>::EPC;
-    constexpr int NW = ElemShape<P, T>::NW;
-    const int rounds = (EPC * S.D + UPW - 1) / UPW, warps = std::max(1, std::min(NW, rounds));
-    const long long groups = (M.E + EPC - 1) / EPC;
-    const int parts = NW == 1 ? factor_parts(groups, rounds) : 1;
-    auto kern = rhs ? factor_elem_kernel<P, T, true> : factor_elem_kernel<P, T, false>;
-    kern<<<(unsigned)(groups * parts), 32 * warps, 0, stream>>>(
-        S.D, M.E, S.member_of, S.faceinfo, S.omega_dev, sigma_t, Mm, Gx, Gy, nds, make_facetab<T>(M.tab),
-        M.nx, M.ny, S.members, (T*)*recp, M.dev_status, piv_count, S.pivot_list, force_pivot, ra, parts);
+  if constexpr (P >= 3) {
+    auto launch = [&](auto kern, long long groups, int parts, int warps) {
+      kern<<<(unsigned)(groups * parts), 32 * warps, 0, stream>>>(
+          S.D, M.E, S.member_of, S.faceinfo, S.omega_dev, sigma_t, Mm, Gx, Gy, nds, make_facetab<T>(M.tab),
+          M.nx, M.ny, S.members, (T*)*recp, M.dev_status, piv_count, S.pivot_list, force_pivot, ra, parts);
+    };
+    auto elem = [&](auto few) {
+      constexpr bool FEW = decltype(few)::value;
+      using Sh = ElemShape<P, T, FEW>;
+      constexpr int UPW = 32 / Sh::LPU;
+      const int rounds = (Sh::EPC * S.D + UPW - 1) / UPW;
+      const long long groups = (M.E + Sh::EPC - 1) / Sh::EPC;
+      launch(rhs ? factor_elem_kernel<P, T, true, FEW> : factor_elem_kernel<P, T, false, FEW>, groups,
+             FEW ? rounds : Sh::NW == 1 ? factor_parts(groups, rounds) : 1, std::max(1, std::min(Sh::NW, rounds)));
+    };
+    if constexpr (sizeof(T) == 4) {
+      elem(std::false_type{});
+    } else if (factor_few<P>(M.E, S.D)) {
+      elem(std::true_type{});
+    } else if constexpr (P == 4) {
+      launch(rhs ? factor_elem4_kernel<true> : factor_elem4_kernel<false>, M.E, factor_parts(M.E, (S.D + 4) / 5), 1);
+    } else {
+      elem(std::false_type{});
+    }
   } else {
     auto kern = rhs ? factor_kernel<P, T, true> : factor_kernel<P, T, false>;
     kern<<<nblk(S.members, 128), 128, 0, stream>>>(
